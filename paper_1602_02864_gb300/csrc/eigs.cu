@@ -15,8 +15,8 @@
 // from S applied to the kept Ritz vectors (whose components orthogonal to V
 // are the residuals).
 //
-// Tall-skinny FP64 kernels: C = A^T B (chunked partials added in a fixed
-// order) and Out = beta Out + alpha A C (one thread per output element).
+// The Krylov-Schur solver's tall-skinny FP64 products, C = A^T B and
+// Out = beta Out + alpha A C, are in tallskinny.cu.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -24,6 +24,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.h"
+#include "tallskinny.h"
 
 namespace spmm {
 
@@ -31,53 +32,147 @@ constexpr int kEigThreads = 256;
 constexpr int kEigMaxBasis = 64;
 constexpr int kTsTile = 16;
 
-// partial[c][r*q + s] = sum over chunk rows i of A[i][r] * B[i][s]
+// ---- the same products in FP64 arithmetic, for the filtered iteration.  A
+// filter of degree 20 multiplies the block's trailing directions' rounding by
+// its own amplification, so there the sums keep their order: products rounded
+// differently in the last place give eigenvectors 1e-4 apart before
+// convergence.  Bound by the FP64 units (two fused multiply-adds per clock and
+// SM), so the work that is known beforehand is left out: half of a symmetric
+// product, all but the diagonal of the residuals', the zero half of an upper
+// triangular factor.
+
+// partial[c][r*q + s] = sum over chunk rows i of A[i][r] * B[i][s]; SYM: A is B
+// (lda == ldb, p == q), only r <= s is summed and its mirror image written.  A
+// thread sums at most NACC elements and loads PER elements of each operand per
+// tile: blocks of up to 16 columns take the small form (40 registers instead
+// of 120, so four blocks an SM instead of two).
+template <bool SYM, int NACC, int PER>
 __global__ void __launch_bounds__(kEigThreads)
-ts_tn_partial_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __restrict__ B, int64_t ldb,
-                     int q, int64_t n, int64_t chunk, double* __restrict__ partial) {
-    __shared__ double ta[kTsTile * kEigMaxBasis];
-    __shared__ double tb[kTsTile * kEigMaxBasis];
-    const int pq = p * q;
+plain_tn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __restrict__ B, int64_t ldb, int q,
+                int64_t n, int64_t chunk, double* __restrict__ partial) {
+    // two tiles: the next one is read into registers while this one is summed
+    __shared__ double ta[2][PER * kEigThreads];
+    __shared__ double tb[2][SYM ? 1 : PER * kEigThreads];
+    const int pq = p * q, ne = SYM ? p * (p + 1) / 2 : pq;
+    // A scheduler's FP64 unit serves its own warps only (warp w: scheduler w % 4),
+    // so the last warps with elements rotate over the schedulers from block to block.
+    const int rot = (int)((blockIdx.x + blockIdx.x / 4) & 3u);
+    const int slot = ((((threadIdx.x >> 5) + rot) << 5) | (threadIdx.x & 31)) & (kEigThreads - 1);
     const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = min(n, i0 + chunk);
-    double acc[16];
+    double acc[NACC];
+    int rs[NACC];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) acc[j] = 0.0;
-    for (int64_t r0 = i0; r0 < i1; r0 += kTsTile) {
+    for (int j = 0; j < NACC; ++j) {
+        acc[j] = 0.0;
+        const int e = slot + j * kEigThreads;
+        int r = e / q, s = e % q;
+        if (SYM && e < ne) {                      // element e of the rows of the upper triangle
+            r = 0;
+            int u = e;
+            while (u >= p - r) u -= p - r, ++r;
+            s = r + u;
+        }
+        rs[j] = r << 8 | s;
+    }
+    double na[PER], nb[PER];
+    auto fetch = [&](int64_t r0) {
         const int rows = (int)min((int64_t)kTsTile, i1 - r0);
-        for (int t = threadIdx.x; t < rows * p; t += blockDim.x) ta[t] = A[(r0 + t / p) * lda + t % p];
-        for (int t = threadIdx.x; t < rows * q; t += blockDim.x) tb[t] = B[(r0 + t / q) * ldb + t % q];
-        __syncthreads();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int e = threadIdx.x + j * kEigThreads;
-            if (e < pq) {
-                const int r = e / q, s = e % q;
-                double f = 0.0;
-                for (int t = 0; t < rows; ++t) f = fma(ta[t * p + r], tb[t * q + s], f);
-                acc[j] += f;
-            }
+        for (int u = 0; u < PER; ++u) {
+            const int t = threadIdx.x + u * kEigThreads;
+            if (t < rows * p) na[u] = A[(r0 + t / p) * lda + t % p];
+            if (!SYM && t < rows * q) nb[u] = B[(r0 + t / q) * ldb + t % q];
+        }
+    };
+    if (i0 < i1) fetch(i0);
+    int buf = 0;
+    for (int64_t r0 = i0; r0 < i1; r0 += kTsTile, buf ^= 1) {
+        const int rows = (int)min((int64_t)kTsTile, i1 - r0);
+        double* sa = ta[buf];
+        double* sb = SYM ? ta[buf] : tb[buf];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int t = threadIdx.x + u * kEigThreads;
+            if (t < rows * p) sa[t] = na[u];
+            if (!SYM && t < rows * q) sb[t] = nb[u];
         }
         __syncthreads();
-    }
+        if (r0 + kTsTile < i1) fetch(r0 + kTsTile);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        const int e = threadIdx.x + j * kEigThreads;
-        if (e < pq) partial[(int64_t)blockIdx.x * pq + e] = acc[j];
+        for (int j = 0; j < NACC; ++j)
+            if (slot + j * kEigThreads < ne) {
+                const int r = rs[j] >> 8, s = rs[j] & 255;
+                double f = 0.0;
+                for (int t = 0; t < rows; ++t) f = fma(sa[t * p + r], sb[t * q + s], f);
+                acc[j] += f;
+            }
     }
+    double* out = partial + (int64_t)blockIdx.x * pq;
+#pragma unroll
+    for (int j = 0; j < NACC; ++j)
+        if (slot + j * kEigThreads < ne) {
+            const int r = rs[j] >> 8, s = rs[j] & 255;
+            out[r * q + s] = acc[j];
+            if (SYM) out[s * q + r] = acc[j];
+        }
 }
 
-__global__ void ts_reduce_kernel(const double* __restrict__ partial, int nparts, int pq, double* __restrict__ out) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < pq; e += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int c = 0; c < nparts; ++c) s += partial[(int64_t)c * pq + e];
-        out[e] = s;
-    }
-}
-
-// Out[i][j] = beta * Out[i][j] + alpha * sum_r A[i][r] * C[r][j]   (C is p x q, row-major)
+// partial[c][j] = sum over chunk rows of (AU - theta U)[i][j]^2: the diagonal of
+// R^T R, each tile of kTsTile rows summed by a thread of its own (column j,
+// tile k of a group), the tiles then added in order.
 __global__ void __launch_bounds__(kEigThreads)
-ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __restrict__ C, int q, double* Out,
-             int64_t ldo, int64_t n, double alpha, double beta) {
+plain_residual_kernel(const double* __restrict__ AU, const double* __restrict__ U, const double* __restrict__ theta,
+                      int q, int64_t n, int64_t chunk, double* __restrict__ partial) {
+    __shared__ double sh[kEigThreads];
+    const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = min(n, i0 + chunk);
+    const int group = kEigThreads / q;            // tiles summed at a time
+    const int j = threadIdx.x % q, k = threadIdx.x / q;
+    double acc = 0.0;
+    for (int64_t g0 = i0; g0 < i1; g0 += (int64_t)group * kTsTile) {
+        double f = 0.0;
+        if (k < group) {
+            const double th = theta[j];
+            const int64_t r0 = g0 + (int64_t)k * kTsTile, r1 = min(i1, r0 + kTsTile);
+            for (int64_t i = r0; i < r1; ++i) {
+                const double r = AU[i * q + j] - th * U[i * q + j];
+                f = fma(r, r, f);
+            }
+        }
+        sh[threadIdx.x] = f;
+        __syncthreads();
+        if (threadIdx.x < q)
+            for (int t = 0; t < group; ++t) acc += sh[t * q + threadIdx.x];
+        __syncthreads();
+    }
+    if (threadIdx.x < q) partial[(int64_t)blockIdx.x * q + threadIdx.x] = acc;
+}
+
+// out[e] = the chunks' partials added in chunk order: a block loads the partials
+// of kReduceElems elements into shared memory at once, then one thread each adds
+// them.
+constexpr int kReduceElems = 4;
+constexpr int kMaxChunks = 1024;
+__global__ void __launch_bounds__(kEigThreads) plain_reduce_kernel(const double* __restrict__ partial, int nparts,
+                                                                   int pq, double* __restrict__ out) {
+    __shared__ double sh[kReduceElems][kMaxChunks];
+    const int e0 = blockIdx.x * kReduceElems;
+    for (int t = threadIdx.x; t < nparts * kReduceElems; t += blockDim.x) {
+        const int c = t / kReduceElems, e = t % kReduceElems;
+        sh[e][c] = e0 + e < pq ? partial[(int64_t)c * pq + e0 + e] : 0.0;
+    }
+    __syncthreads();
+    if (threadIdx.x < kReduceElems && e0 + (int)threadIdx.x < pq) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int c = 0; c < nparts; ++c) s += sh[threadIdx.x][c];
+        out[e0 + threadIdx.x] = s;
+    }
+}
+
+// Out[i][j] = sum_r A[i][r] * C[r][j], r in order (C p x q, row-major)
+__global__ void __launch_bounds__(kEigThreads)
+plain_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __restrict__ C, int q, double* Out,
+                int64_t ldo, int64_t n) {
     __shared__ double cs[kEigMaxBasis * kEigMaxBasis];
     for (int t = threadIdx.x; t < p * q; t += blockDim.x) cs[t] = C[t];
     __syncthreads();
@@ -87,7 +182,37 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
         const int j = (int)(t % q);
         double s = 0.0;
         for (int r = 0; r < p; ++r) s = fma(A[i * lda + r], cs[r * q + j], s);
-        Out[i * ldo + j] = (beta == 0.0 ? 0.0 : beta * Out[i * ldo + j]) + alpha * s;
+        Out[i * ldo + j] = s;
+    }
+}
+
+// The same with C upper triangular (q == p): the terms r > j are zero.  A warp
+// takes 32 rows of one column at a time, so its lanes run equally long, and
+// columns w, q-1-w of each tile in turn, so the warps do too; rows pass
+// through shared memory both ways.
+__global__ void __launch_bounds__(kEigThreads)
+plain_nn_upper_kernel(const double* __restrict__ A, const double* __restrict__ C, int q, double* __restrict__ Out,
+                      int64_t n) {
+    extern __shared__ double ts_sh[];
+    const int ld = q | 1;                         // odd row stride: no bank conflicts between rows
+    double *cs = ts_sh, *a = cs + q * q, *o = a + 32 * ld;
+    for (int t = threadIdx.x; t < q * q; t += blockDim.x) cs[t] = C[t];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kEigThreads / 32;
+    for (int64_t r0 = (int64_t)blockIdx.x * 32; r0 < n; r0 += (int64_t)gridDim.x * 32) {
+        const int rows = (int)min((int64_t)32, n - r0);
+        __syncthreads();
+        for (int t = threadIdx.x; t < rows * q; t += blockDim.x) a[(t / q) * ld + t % q] = A[r0 * q + t];
+        __syncthreads();
+        for (int h = warp; 2 * h < q; h += nw)
+            for (int side = 0; side < 2; ++side) {
+                const int j = side ? q - 1 - h : h;
+                if (side && j == h) break;
+                double s = 0.0;
+                for (int r = 0; r <= j; ++r) s = fma(a[lane * ld + r], cs[r * q + j], s);
+                o[lane * ld + j] = s;
+            }
+        __syncthreads();
+        for (int t = threadIdx.x; t < rows * q; t += blockDim.x) Out[r0 * q + t] = o[(t / q) * ld + t % q];
     }
 }
 
@@ -116,14 +241,6 @@ __global__ void copy_block_kernel(const double* __restrict__ src, int64_t lds, i
         dst[(t / b) * ldd + t % b] = src[(t / b) * lds + t % b];
 }
 
-// residual block R = AU - U diag(theta)
-__global__ void residual_kernel(const double* __restrict__ AU, const double* __restrict__ U, const double* theta,
-                                int q, int64_t n, double* R) {
-    const int64_t total = n * q;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x)
-        R[t] = AU[t] - theta[t % q] * U[t];
-}
-
 // Chebyshev filter step (FP32): Yn = alpha * SY + beta * Yc + gamma * Yp,
 // coefficients (alpha, beta, gamma) read from device memory so one captured
 // graph serves every filter interval
@@ -141,54 +258,88 @@ __global__ void f32_to_bf16_kernel(const float* __restrict__ src, int64_t total,
         dst[t] = __float2bfloat16(src[t]);
 }
 
-// Block Cholesky G = R^T R (R upper, b x b row-major, b <= 32) and its inverse
-// Rinv = R^-1 (upper), by one block of 32 threads: the pivots in turn (thread
-// 0), each pivot's row of R across the threads, then column c of the inverse
-// by back substitution in thread c.  A pivot that is not safely positive
-// (below 1e-24 x trace) marks *flag and leaves the identity in Rinv, so the
-// kernels queued after it keep running on finite numbers until the host
-// reads the flag.
-__global__ void chol_inv_kernel(const double* __restrict__ G, int b, double* __restrict__ Rinv,
-                                int32_t* __restrict__ flag) {
-    __shared__ double R[32 * 32];
-    __shared__ int bad;
+// 1 / sqrt(d) for a positive normal d: the FP32 value of d scaled by a power of
+// four to [1, 4), refined twice (y += y (1 - d y^2) / 2; relative error 1e-7,
+// 1e-14, then the rounding of the last step).
+__device__ __forceinline__ double rsqrt_newton(double d) {
+    const int hi = __double2hiint(d), e = ((hi >> 20) - 1023) & ~1;
+    const double m = __hiloint2double(hi - (e << 20), __double2loint(d));
+    double y = (double)rsqrtf((float)m);
+    const double half = 0.5 * m;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const double r = fma(-half * y, y, 0.5);
+        y = fma(y, r, y);
+    }
+    return __hiloint2double(__double2hiint(y) - ((e / 2) << 20), __double2loint(y));
+}
+
+// Block Cholesky G = R^T R (R upper, b x b row-major, b <= B <= 32) and its
+// inverse Rinv = R^-1 (upper), by one warp: lane i holds column i in registers,
+// a pivot's row is passed by shuffles and its multiples are subtracted from the
+// rows below (the same differences in the same order as the left-looking
+// form); then lane c builds column c of the inverse by back substitution, row
+// by row.  Bound by its FP64 instructions, 64 clocks each on one scheduler, so
+// a pivot costs one reciprocal square root (FP32 and two Newton steps) instead
+// of a square root and two divisions.  A pivot that is not
+// safely positive (below 1e-24 x trace) marks *flag and leaves the identity in
+// Rinv, so the kernels queued after it keep running on finite numbers until the
+// host reads the flag.
+template <int B>
+__global__ void __launch_bounds__(32) chol_inv_kernel(const double* __restrict__ G, int b, double* __restrict__ Rinv,
+                                                      int32_t* __restrict__ flag) {
+    __shared__ double R[B * B];
     const int t = threadIdx.x;
-    if (t == 0) bad = 0;
-    for (int e = t; e < b * b; e += blockDim.x) R[e] = 0.0;
-    __syncthreads();
+    double a[B];
     double tr = 0.0;
     for (int i = 0; i < b; ++i) tr += G[i * b + i];
-    for (int j = 0; j < b; ++j) {
-        if (t == 0) {
-            double d = G[j * b + j];
-            for (int k = 0; k < j; ++k) d -= R[k * b + j] * R[k * b + j];
-            if (!(d > 1e-24 * (tr > 0 ? tr : 1.0))) bad = 1;
-            R[j * b + j] = bad ? 1.0 : sqrt(d);
+    const double floor_d = 1e-24 * (tr > 0 ? tr : 1.0);
+#pragma unroll
+    for (int k = 0; k < B; ++k) a[k] = (t < b && k <= t) ? G[k * b + t] : 0.0;
+    double rdiag = 1.0;                          // 1 / R[t][t]
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < B; ++j) {
+        if (j < b && !bad) {
+            const double d = __shfl_sync(0xffffffffu, a[j], j);
+            bad = !(d > floor_d);
+            if (!bad) {
+                const double y = rsqrt_newton(d);
+                a[j] *= y;                       // lane j: sqrt(d)
+                if (t == j) rdiag = y;
+                if (t < b) R[j * B + t] = t >= j ? a[j] : 0.0;
+#pragma unroll
+                for (int k = j + 1; k < B; ++k)
+                    if (k < b) {
+                        const double rjk = __shfl_sync(0xffffffffu, a[j], k);
+                        if (k <= t) a[k] = fma(-rjk, a[j], a[k]);
+                    }
+            }
         }
-        __syncthreads();
-        if (bad) break;
-        const double rjj = R[j * b + j];
-        for (int i = j + 1 + t; i < b; i += blockDim.x) {
-            double s = G[j * b + i];
-            for (int k = 0; k < j; ++k) s -= R[k * b + j] * R[k * b + i];
-            R[j * b + i] = s / rjj;
-        }
-        __syncthreads();
     }
     if (bad) {
-        for (int e = t; e < b * b; e += blockDim.x) Rinv[e] = (e / b == e % b) ? 1.0 : 0.0;
+        for (int e = t; e < b * b; e += 32) Rinv[e] = (e / b == e % b) ? 1.0 : 0.0;
         if (t == 0) *flag = 1;
         return;
     }
-    for (int c = t; c < b; c += blockDim.x) {
-        double x[32];
-        x[c] = 1.0 / R[c * b + c];
-        for (int i = c - 1; i >= 0; --i) {
-            double s = 0.0;
-            for (int k = i + 1; k <= c; ++k) s += R[i * b + k] * x[k];
-            x[i] = -s / R[i * b + i];
+    __syncwarp();
+    double x[B];
+#pragma unroll
+    for (int i = B - 1; i >= 0; --i) {
+        x[i] = 0.0;
+        if (i < b) {
+            double s0 = 0.0, s1 = 0.0;           // x[k] = 0 below the diagonal of column t
+#pragma unroll
+            for (int k = i + 1; k < B; ++k)
+                if (k < b) {
+                    if (k & 1) s1 = fma(R[i * B + k], x[k], s1);
+                    else s0 = fma(R[i * B + k], x[k], s0);
+                }
+            const double ri = __shfl_sync(0xffffffffu, rdiag, i);
+            if (i == t) x[i] = ri;
+            else if (i < t) x[i] = -(s0 + s1) * ri;
+            if (t < b) Rinv[i * b + t] = x[i];
         }
-        for (int i = 0; i < b; ++i) Rinv[i * b + c] = i <= c ? x[i] : 0.0;
     }
 }
 
@@ -285,25 +436,57 @@ struct Eig {
     int32_t* flags = nullptr;   // breakdown flag of each expansion of a cycle (device)
     float* Yf = nullptr;
     void* Xs = nullptr;
-    int64_t chunk = 0;
+    bool plain = false;         // the products in FP64 arithmetic (filtered iteration)
+    int64_t chunk = 0;          // rows per partial of the plain products
     int nchunks = 0;
     int grid = 0;
 
+    // C = A^T B on the host
     cudaError_t tn(const double* Am, int64_t lda, int p, const double* Bm, int64_t ldb, int q, std::vector<double>& out) {
-        ts_tn_partial_kernel<<<nchunks, kEigThreads, 0, s>>>(Am, lda, p, Bm, ldb, q, n, chunk, part);
-        ts_reduce_kernel<<<(p * q + 255) / 256, 256, 0, s>>>(part, nchunks, p * q, small);
-        out.resize((size_t)p * q);
-        cudaError_t e = cudaMemcpyAsync(out.data(), small, (size_t)p * q * sizeof(double), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        return e;
+        cudaError_t e = cudaSuccess;
+        if (!plain) {
+            e = ts_tn(Am, lda, p, Bm, ldb, q, n, part, small, s);
+        } else {
+            const bool sym = Am == Bm && lda == ldb && p == q, narrow = p <= 16 && q <= 16;
+            auto kernel = narrow ? (sym ? plain_tn_kernel<true, 1, 1> : plain_tn_kernel<false, 1, 1>)
+                                 : (sym ? plain_tn_kernel<true, 16, 4> : plain_tn_kernel<false, 16, 4>);
+            kernel<<<nchunks, kEigThreads, 0, s>>>(Am, lda, p, Bm, ldb, q, n, chunk, part);
+            plain_reduce_kernel<<<(p * q + kReduceElems - 1) / kReduceElems, kEigThreads, 0, s>>>(part, nchunks, p * q, small);
+        }
+        return download(p * q, out, e);
     }
+    // Out = A C (C from the host; upper: C is upper triangular and A, Out are contiguous)
     cudaError_t nn(const double* Am, int64_t lda, int p, const std::vector<double>& C, int q, double* Out, int64_t ldo,
-                   double alpha, double beta) {
+                   bool upper = false) {
         cudaError_t e = cudaMemcpyAsync(small, C.data(), (size_t)p * q * sizeof(double), cudaMemcpyHostToDevice, s);
-        if (e != cudaSuccess) return e;
-        ts_nn_kernel<<<grid, kEigThreads, 0, s>>>(Am, lda, p, small, q, Out, ldo, n, alpha, beta);
+        if (e == cudaSuccess && !plain) e = ts_nn(Am, lda, p, small, q, Out, ldo, n, 1.0, 0.0, s);
+        if (e == cudaSuccess && plain) {
+            const size_t smem = ((size_t)q * q + 64 * (size_t)(q | 1)) * sizeof(double);
+            if (upper && smem <= 48 * 1024)
+                plain_nn_upper_kernel<<<grid, kEigThreads, smem, s>>>(Am, small, q, Out, n);
+            else
+                plain_nn_kernel<<<grid, kEigThreads, 0, s>>>(Am, lda, p, small, q, Out, ldo, n);
+        }
         // small is reused by the next call: finish this one first
-        return cudaStreamSynchronize(s);
+        return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+    }
+    // squared residual norms of q Ritz pairs (theta on the host)
+    cudaError_t residuals(const double* AUm, const double* Um, const std::vector<double>& th, int q,
+                          std::vector<double>& out) {
+        cudaError_t e = cudaMemcpyAsync(theta, th.data(), (size_t)q * sizeof(double), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess && !plain) e = ts_residuals(AUm, Um, theta, q, n, part, small, s);
+        if (e == cudaSuccess && plain) {
+            plain_residual_kernel<<<nchunks, kEigThreads, 0, s>>>(AUm, Um, theta, q, n, chunk, part);
+            plain_reduce_kernel<<<(q + kReduceElems - 1) / kReduceElems, kEigThreads, 0, s>>>(part, nchunks, q, small);
+        }
+        return download(q, out, e);
+    }
+    cudaError_t download(int count, std::vector<double>& out, cudaError_t e) {
+        out.resize((size_t)count);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(out.data(), small, (size_t)count * sizeof(double), cudaMemcpyDeviceToHost, s);
+        return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
     }
     // Y = S * block (block: n x b FP64 with leading dimension ld) into out (ld m)
     int apply_block(const double* blk, int64_t ld, double* out, int64_t ldo) {
@@ -319,30 +502,23 @@ struct Eig {
         f32_to_f64_kernel<<<grid, kEigThreads, 0, s>>>(Yf, b, n, out, ldo);
         return SPMM_OK;
     }
-    // C = A^T B into device memory, and Out = beta Out + alpha A C with C in
-    // device memory: the tall-skinny products with no host round trip
-    void tn_dev(const double* Am, int64_t lda, int p, const double* Bm, int64_t ldb, int q, double* out) {
-        ts_tn_partial_kernel<<<nchunks, kEigThreads, 0, s>>>(Am, lda, p, Bm, ldb, q, n, chunk, part);
-        ts_reduce_kernel<<<(p * q + 255) / 256, 256, 0, s>>>(part, nchunks, p * q, out);
-    }
-    void nn_dev(const double* Am, int64_t lda, int p, const double* C, int q, double* Out, int64_t ldo, double alpha,
-                double beta) {
-        ts_nn_kernel<<<grid, kEigThreads, 0, s>>>(Am, lda, p, C, q, Out, ldo, n, alpha, beta);
-    }
     // orthonormalise() on the device only: CGS2 against V[:, :cur], then
     // CholQR2 with the Cholesky factor inverted by chol_inv_kernel; a
     // breakdown marks flags[slot] instead of returning
-    void orthonormalize_dev(int cur, int slot) {
-        for (int pass = 0; pass < 2 && cur > 0; ++pass) {
-            tn_dev(V, m, cur, W, b, b, small);
-            nn_dev(V, m, cur, small, b, W, b, -1.0, 1.0);
+    cudaError_t orthonormalize_dev(int cur, int slot) {
+        cudaError_t e = cudaSuccess;
+        for (int pass = 0; pass < 2 && cur > 0 && e == cudaSuccess; ++pass) {
+            e = ts_tn(V, m, cur, W, b, b, n, part, small, s);
+            if (e == cudaSuccess) e = ts_nn(V, m, cur, small, b, W, b, n, -1.0, 1.0, s);
         }
-        for (int pass = 0; pass < 2; ++pass) {
-            tn_dev(W, b, b, W, b, b, small);
-            chol_inv_kernel<<<1, 32, 0, s>>>(small, b, small2, flags + slot);
-            nn_dev(W, b, b, small2, b, W2, b, 1.0, 0.0);
+        for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+            if ((e = ts_tn(W, b, b, W, b, b, n, part, small, s)) != cudaSuccess) break;
+            if (b <= 16) chol_inv_kernel<16><<<1, 32, 0, s>>>(small, b, small2, flags + slot);
+            else chol_inv_kernel<32><<<1, 32, 0, s>>>(small, b, small2, flags + slot);
+            e = ts_nn(W, b, b, small2, b, W2, b, n, 1.0, 0.0, s);
             std::swap(W, W2);
         }
+        return e;
     }
     // n_exp expansions of the basis from column cur0, the first from the
     // image AV[:, seed0] and each next one from the image of the block before;
@@ -354,7 +530,7 @@ struct Eig {
         int cur = cur0, seed = seed0;
         for (int x = 0; x < n_exp; ++x) {
             copy_block_kernel<<<grid, kEigThreads, 0, s>>>(AV + seed, m, b, n, W, b);
-            orthonormalize_dev(cur, x);
+            if ((e = orthonormalize_dev(cur, x)) != cudaSuccess) return cuda_fail(e, "spmm_eigs: orthonormalise");
             copy_block_kernel<<<grid, kEigThreads, 0, s>>>(W, b, b, n, V + cur, m);
             const int rc = apply_block(V + cur, m, AV + cur, m);
             if (rc != SPMM_OK) return rc;
@@ -364,18 +540,14 @@ struct Eig {
         e = cudaGetLastError();
         return e == cudaSuccess ? SPMM_OK : cuda_fail(e, "spmm_eigs: expansion");
     }
-    // orthonormalise W (n x b) against V[:, :cur] twice, then CholQR2; false on breakdown
-    bool orthonormalize(int cur, cudaError_t& e) {
-        std::vector<double> C, G, R;
-        for (int pass = 0; pass < 2 && cur > 0; ++pass) {
-            if ((e = tn(V, m, cur, W, b, b, C)) != cudaSuccess) return false;
-            if ((e = nn(V, m, cur, C, b, W, b, -1.0, 1.0)) != cudaSuccess) return false;
-        }
+    // orthonormalise W (n x b) by CholQR2; false on breakdown
+    bool orthonormalize(cudaError_t& e) {
+        std::vector<double> G, R;
         for (int pass = 0; pass < 2; ++pass) {
             if ((e = tn(W, b, b, W, b, b, G)) != cudaSuccess) return false;
             if (!cholesky_upper(b, G, R)) return false;
             const std::vector<double> Ri = upper_inverse(b, R);
-            if ((e = nn(W, b, b, Ri, b, W2, b, 1.0, 0.0)) != cudaSuccess) return false;
+            if ((e = nn(W, b, b, Ri, b, W2, b, true)) != cudaSuccess) return false;
             std::swap(W, W2);
         }
         return true;
@@ -418,8 +590,6 @@ static int eigs_impl(spmm_mat_t S, int op, int32_t nev, int32_t block, int32_t m
     E.xtype = xtype;
     E.op = op;
     E.grid = std::max(1, sms * 8);
-    E.chunk = std::max<int64_t>(1024, (n + 1023) / 1024);
-    E.nchunks = (int)((n + E.chunk - 1) / E.chunk);
     const int m = max_basis, b = block;
     const int keep = std::min(nev + b, m - b);
     int rc = SPMM_OK;
@@ -431,9 +601,9 @@ static int eigs_impl(spmm_mat_t S, int op, int32_t nev, int32_t block, int32_t m
         const size_t nm = (size_t)n * m * sizeof(double);
         if ((e = cudaMalloc((void**)&E.V, nm)) != cudaSuccess || (e = cudaMalloc((void**)&E.AV, nm)) != cudaSuccess ||
             (e = cudaMalloc((void**)&E.U, nm)) != cudaSuccess || (e = cudaMalloc((void**)&E.AU, nm)) != cudaSuccess ||
-            (e = cudaMalloc((void**)&E.W, (size_t)n * m * sizeof(double))) != cudaSuccess ||
-            (e = cudaMalloc((void**)&E.W2, (size_t)n * m * sizeof(double))) != cudaSuccess ||
-            (e = cudaMalloc((void**)&E.part, (size_t)E.nchunks * m * m * sizeof(double))) != cudaSuccess ||
+            (e = cudaMalloc((void**)&E.W, (size_t)n * b * sizeof(double))) != cudaSuccess ||
+            (e = cudaMalloc((void**)&E.W2, (size_t)n * b * sizeof(double))) != cudaSuccess ||
+            (e = cudaMalloc((void**)&E.part, ts_partial_doubles(n, m) * sizeof(double))) != cudaSuccess ||
             (e = cudaMalloc((void**)&E.small, (size_t)m * m * sizeof(double))) != cudaSuccess ||
             (e = cudaMalloc((void**)&E.small2, (size_t)b * b * sizeof(double))) != cudaSuccess ||
             (e = cudaMalloc((void**)&E.flags, (size_t)kEigMaxBasis * sizeof(int32_t))) != cudaSuccess ||
@@ -447,7 +617,7 @@ static int eigs_impl(spmm_mat_t S, int op, int32_t nev, int32_t block, int32_t m
         }
         // start block
         copy_block_kernel<<<E.grid, kEigThreads, 0, E.s>>>(V0, b, b, n, E.W, b);
-        if (!E.orthonormalize(0, e)) {
+        if (!E.orthonormalize(e)) {
             if (e != cudaSuccess) fail(e, "spmm_eigs: orthonormalise");
             else { set_error("spmm_eigs: the start block is rank-deficient"); rc = SPMM_ERR_ARG; }
             break;
@@ -525,21 +695,19 @@ static int eigs_impl(spmm_mat_t S, int op, int32_t nev, int32_t block, int32_t m
                 thk[c] = th[order[c]];
                 for (int r = 0; r < cur; ++r) Yk[(size_t)r * kp + c] = Y[(size_t)r * cur + order[c]];
             }
-            if ((e = E.nn(E.V, m, cur, Yk, kp, E.U, kp, 1.0, 0.0)) != cudaSuccess ||
-                (e = E.nn(E.AV, m, cur, Yk, kp, E.AU, kp, 1.0, 0.0)) != cudaSuccess) {
+            if ((e = E.nn(E.V, m, cur, Yk, kp, E.U, kp)) != cudaSuccess ||
+                (e = E.nn(E.AV, m, cur, Yk, kp, E.AU, kp)) != cudaSuccess) {
                 fail(e, "spmm_eigs: Ritz vectors");
                 break;
             }
             // residual norms of the Ritz pairs
-            cudaMemcpyAsync(E.theta, thk.data(), kp * sizeof(double), cudaMemcpyHostToDevice, E.s);
-            residual_kernel<<<E.grid, kEigThreads, 0, E.s>>>(E.AU, E.U, E.theta, kp, n, E.W2);
-            if ((e = E.tn(E.W2, kp, kp, E.W2, kp, kp, Rn)) != cudaSuccess) { fail(e, "spmm_eigs: residuals"); break; }
+            if ((e = E.residuals(E.AU, E.U, thk, kp, Rn)) != cudaSuccess) { fail(e, "spmm_eigs: residuals"); break; }
             double worst = 0.0;
-            for (int i = 0; i < nev; ++i) worst = std::max(worst, std::sqrt(std::max(0.0, Rn[(size_t)i * kp + i])));
+            for (int i = 0; i < nev; ++i) worst = std::max(worst, std::sqrt(std::max(0.0, Rn[(size_t)i])));
             if (worst <= tol || restarts >= max_restarts) {
                 for (int i = 0; i < nev; ++i) {
                     evals[i] = thk[i];
-                    if (resid) resid[i] = std::sqrt(std::max(0.0, Rn[(size_t)i * kp + i]));
+                    if (resid) resid[i] = std::sqrt(std::max(0.0, Rn[(size_t)i]));
                 }
                 if (evecs) copy_block_kernel<<<E.grid, kEigThreads, 0, E.s>>>(E.U, kp, nev, n, evecs, nev);
                 if (restarts_out) *restarts_out = restarts;
@@ -670,8 +838,9 @@ static int eigs_filtered_impl(spmm_mat_t S, int32_t nev, int32_t block, int32_t 
     // rounding of U
     E.xtype = S->vtype == SPMM_BF16 ? SPMM_BF16 : SPMM_F32;
     E.grid = std::max(1, sms * 8);
-    E.chunk = std::max<int64_t>(1024, (n + 1023) / 1024);
-    E.nchunks = (int)((n + E.chunk - 1) / E.chunk);
+    E.plain = true;
+    E.chunk = std::max<int64_t>(1024, (n + kMaxChunks - 1) / kMaxChunks);
+    E.nchunks = (int)((n + E.chunk - 1) / E.chunk);   // at most kMaxChunks
     float* Yc[3] = {nullptr, nullptr, nullptr};
     float* coef = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -700,7 +869,7 @@ static int eigs_filtered_impl(spmm_mat_t S, int32_t nev, int32_t block, int32_t 
         }
         // U = orthonormalised start block; SU = S U; Rayleigh-Ritz
         copy_block_kernel<<<E.grid, kEigThreads, 0, E.s>>>(V0, b, b, n, E.W, b);
-        if (!E.orthonormalize(0, e)) {
+        if (!E.orthonormalize(e)) {
             if (e != cudaSuccess) fail(e, "spmm_eigs_filtered: orthonormalise");
             else { set_error("spmm_eigs_filtered: the start block is rank-deficient"); rc = SPMM_ERR_ARG; }
             break;
@@ -727,18 +896,16 @@ static int eigs_filtered_impl(spmm_mat_t S, int32_t nev, int32_t block, int32_t 
                 for (int r = 0; r < b; ++r) Yk[(size_t)r * b + c] = Y[(size_t)r * b + order[c]];
             }
             // Ritz vectors and their images; residual norms
-            if ((e = E.nn(E.V, b, b, Yk, b, E.U, b, 1.0, 0.0)) != cudaSuccess ||
-                (e = E.nn(E.AV, b, b, Yk, b, E.AU, b, 1.0, 0.0)) != cudaSuccess) {
+            if ((e = E.nn(E.V, b, b, Yk, b, E.U, b)) != cudaSuccess ||
+                (e = E.nn(E.AV, b, b, Yk, b, E.AU, b)) != cudaSuccess) {
                 fail(e, "spmm_eigs_filtered: Ritz vectors");
                 break;
             }
             std::swap(E.V, E.U);
             std::swap(E.AV, E.AU);
-            cudaMemcpyAsync(E.theta, thk.data(), b * sizeof(double), cudaMemcpyHostToDevice, E.s);
-            residual_kernel<<<E.grid, kEigThreads, 0, E.s>>>(E.AV, E.V, E.theta, b, n, E.W2);
-            if ((e = E.tn(E.W2, b, b, E.W2, b, b, Rn)) != cudaSuccess) { fail(e, "spmm_eigs_filtered: residuals"); break; }
+            if ((e = E.residuals(E.AV, E.V, thk, b, Rn)) != cudaSuccess) { fail(e, "spmm_eigs_filtered: residuals"); break; }
             double worst = 0.0;
-            for (int i = 0; i < b; ++i) best_res[i] = std::sqrt(std::max(0.0, Rn[(size_t)i * b + i]));
+            for (int i = 0; i < b; ++i) best_res[i] = std::sqrt(std::max(0.0, Rn[(size_t)i]));
             for (int i = 0; i < nev; ++i) worst = std::max(worst, best_res[i]);
             if (worst <= tol || it >= max_iters) break;
             // ---- filter the block: coefficients for this interval
@@ -808,7 +975,7 @@ static int eigs_filtered_impl(spmm_mat_t S, int32_t nev, int32_t block, int32_t 
             if ((e = cudaGraphLaunch(exec, E.s)) != cudaSuccess) { fail(e, "spmm_eigs_filtered: filter"); break; }
             // the filtered block, orthonormalised, is the next U
             f32_to_f64_kernel<<<E.grid, kEigThreads, 0, E.s>>>(Yc[degree % 3], b, n, E.W, b);
-            if (!E.orthonormalize(0, e)) {
+            if (!E.orthonormalize(e)) {
                 if (e != cudaSuccess) fail(e, "spmm_eigs_filtered: orthonormalise");
                 else {
                     set_error("spmm_eigs_filtered: the filtered block lost rank (lower the degree)");

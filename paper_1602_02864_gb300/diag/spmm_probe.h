@@ -1,4 +1,4 @@
-// spmm_probe.h -- gather-rate diagnostics, built as libspmm_probe.so
+// spmm_probe.h -- diagnostics (gather rates, the eigensolvers' FP64 products), built as libspmm_probe.so
 // beside libspmm.so (which it links against for the handle and its error
 // string).  Not part of the library's interface and not a paper operation:
 // they measure the rate of random row gathers, the SpMM's dominant cost, as
@@ -39,6 +39,18 @@ int spmm_probe_gather(int64_t table_bytes, int32_t row_bytes, double* rows_per_s
  */
 int spmm_probe_gather_cols(spmm_mat_t A, int32_t transpose, int32_t row_bytes, double* rows_per_s,
                            double* bytes_per_s, void* stream);
+
+/*
+ * spmm_probe_ts_tn, spmm_probe_ts_nn -- diagnostic: the eigensolvers' FP64
+ * products of tall, narrow matrices on device arrays, to check their accuracy
+ * by themselves: C (p x q) = A^T B with A n x p, B n x q, and
+ * Out (n x q) = beta Out + alpha A C; 1 <= p, q <= 64, n >= 1.
+ * Synchronise `stream`; allocate scratch.
+ */
+int spmm_probe_ts_tn(const double* A, int64_t lda, int32_t p, const double* B, int64_t ldb, int32_t q, int64_t n,
+                     double* C, void* stream);
+int spmm_probe_ts_nn(const double* A, int64_t lda, int32_t p, const double* C, int32_t q, double* Out, int64_t ldo,
+                     int64_t n, double alpha, double beta, void* stream);
 
 #ifdef __cplusplus
 }
