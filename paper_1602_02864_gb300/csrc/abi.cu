@@ -657,10 +657,10 @@ extern "C" int spmm_create_batched(spmm_mat_t* out, int32_t n_graphs, const int6
 namespace spmm {
 
 // The task counter of a launch (reset on s) and the tasks claimed at a time.
-unsigned long long* task_counter(const DevCSR& d, int32_t k, int32_t xtype, cudaStream_t s, cudaError_t* e,
-                                 int32_t* chunk) {
+unsigned long long* task_counter(const DevCSR& d, int64_t n_tasks, int32_t k, int32_t xtype, cudaStream_t s,
+                                 cudaError_t* e, int32_t* chunk) {
     *e = cudaSuccess;
-    *chunk = (int64_t)k * (int64_t)dtype_size((spmm_dtype)xtype) >= kWideRowBytes ? 1 : kNarrowTaskChunk;
+    *chunk = claim_chunk(n_tasks, (int64_t)k * (int64_t)dtype_size((spmm_dtype)xtype) >= kWideRowBytes);
     if (!d.task_ctr) return nullptr;
     *e = cudaMemsetAsync(d.task_ctr, 0, sizeof(unsigned long long), s);
     return *e == cudaSuccess ? d.task_ctr : nullptr;
@@ -714,6 +714,7 @@ void set_geometry(FwdArgs& a, const void* X, int64_t ldx, int32_t k, int32_t xty
                      : d.short_runs == 1 ? false
                                          : pieces_ok && (lg >= 2 || vec * esize <= 8) &&
                                                d.walk_eff[4 - lg] < kPiecesBelowWalkEff;
+    a.x_large = d.n_cols * ldx * esize > kLargeXBytes;
     *vec_out = vec;
     *ch_out = ch;
 }
@@ -727,10 +728,19 @@ int value_mode(const spmm_mat* A, int32_t xtype) {
     return vmode;
 }
 
-cudaError_t launch_rows(const FwdArgs& a, int32_t xtype, int vmode, int vec, int ch, cudaStream_t s) {
-    if (xtype == SPMM_F32) return launch_rows_f32(a, vmode, vec, ch, s);
-    if (xtype == SPMM_BF16) return launch_rows_bf16(a, vmode, vec, ch, s);
-    return launch_rows_f16(a, vmode, vec, ch, s);
+cudaError_t launch_rows(const FwdArgs& all, int32_t xtype, int vmode, int vec, int ch, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    // the kernel numbers a launch's tasks in 32 bits; parts after the first take the static schedule
+    for (int64_t t0 = 0; t0 < all.n_tasks && e == cudaSuccess; t0 += kMaxLaunchTasks) {
+        FwdArgs a = all;
+        a.tasks = all.tasks + t0;
+        a.n_tasks = std::min(kMaxLaunchTasks, all.n_tasks - t0);
+        if (t0 > 0) a.task_ctr = nullptr;
+        if (xtype == SPMM_F32) e = launch_rows_f32(a, vmode, vec, ch, s);
+        else if (xtype == SPMM_BF16) e = launch_rows_bf16(a, vmode, vec, ch, s);
+        else e = launch_rows_f16(a, vmode, vec, ch, s);
+    }
+    return e;
 }
 
 // The product on a resident handle: one run over all tasks (rows_done ==
@@ -780,7 +790,7 @@ static int apply_resident(const spmm_mat* A, int transpose, const void* X, int64
     for (size_t j = 0; j < n_runs; ++j) {
         const RowBlock& b = by_runs ? d.row_blocks[j] : all;
         cudaError_t ec = cudaSuccess;
-        a.task_ctr = task_counter(d, k, xtype, s, &ec, &a.task_chunk);
+        a.task_ctr = task_counter(d, b.t1 - b.t0, k, xtype, s, &ec, &a.task_chunk);
         if (ec != cudaSuccess) return cuda_fail(ec, "spmm_apply: task counter");
         a.tasks = d.tasks + b.t0;
         a.n_tasks = b.t1 - b.t0;

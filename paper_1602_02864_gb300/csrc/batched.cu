@@ -49,6 +49,8 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
         int vmode, vec, ch;
         bool comp;
         LaneGeometry gm;
+        int64_t t0 = 0;             // first task (of at most kMaxLaunchTasks)
+        int64_t tasks() const { return std::min(kMaxLaunchTasks, d->n_tasks - t0); }
     };
     std::map<std::tuple<int, int, int, int>, std::vector<Entry>> groups;
     std::vector<Entry> all;
@@ -91,9 +93,13 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
     // ---- one launch per group (and per kMaxBatch entries of it)
     auto M = std::make_unique<MultiArgs>();
     for (auto& kv : groups) {
-        const std::vector<Entry>& es = kv.second;
-        for (size_t c0 = 0; c0 < es.size(); c0 += kMaxBatch) {
-            const size_t c1 = std::min(es.size(), c0 + (size_t)kMaxBatch);
+        std::vector<Entry> es;      // an entry with more tasks than a launch takes comes in pieces
+        for (Entry en : kv.second)
+            for (en.t0 = 0; en.t0 < en.d->n_tasks; en.t0 += kMaxLaunchTasks) es.push_back(en);
+        for (size_t c0 = 0, c1 = 0; c0 < es.size(); c0 = c1) {
+            int64_t room = kMaxLaunchTasks;
+            for (c1 = c0; c1 < es.size() && c1 < c0 + (size_t)kMaxBatch && es[c1].tasks() <= room; ++c1)
+                room -= es[c1].tasks();
             *M = MultiArgs{};
             M->n = (int32_t)(c1 - c0);
             int64_t tot = 0;
@@ -107,8 +113,8 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
                 a.row_ptr = d.row_ptr;
                 a.col_idx = d.col_idx;
                 a.val = d.val;
-                a.tasks = d.tasks;
-                a.n_tasks = d.n_tasks;
+                a.tasks = d.tasks + en.t0;
+                a.n_tasks = en.tasks();
                 a.partials = d.partials;
                 a.n_slots = d.n_slots;
                 a.X = X[en.i];
@@ -124,7 +130,7 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
                 a.compensated = en.comp ? 1 : 0;
                 a.partials_comp = d.partials_comp;
                 M->off[q - c0] = tot;
-                tot += d.n_tasks;
+                tot += en.tasks();
                 wide = wide || (int64_t)k[en.i] * esize >= kWideRowBytes;
             }
             M->off[M->n] = tot;
@@ -133,7 +139,7 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
             M->g.n_tasks = tot;
             M->g.status = A[first.i]->status;
             M->g.wait_ns = kWaitNs;
-            M->g.task_chunk = wide ? 1 : kNarrowTaskChunk;
+            M->g.task_chunk = claim_chunk(tot, wide);
             M->g.task_ctr = first.d->task_ctr;
             cudaError_t e = cudaSuccess;
             if (M->g.task_ctr) e = cudaMemsetAsync(M->g.task_ctr, 0, sizeof(unsigned long long), s);

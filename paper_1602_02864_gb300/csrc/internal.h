@@ -294,8 +294,8 @@ int apply_dev_runs(const spmm_mat* A, int transpose, const void* X, int64_t ldx,
                    int64_t ldy, cudaStream_t s, const std::function<int(int64_t, int64_t)>& rows_done);
 // the task counter for a launch over rows of k elements of xtype (reset on s;
 // nullptr for the static schedule) and the number of tasks per claim
-unsigned long long* task_counter(const DevCSR& d, int32_t k, int32_t xtype, cudaStream_t s, cudaError_t* e,
-                                 int32_t* chunk);
+unsigned long long* task_counter(const DevCSR& d, int64_t n_tasks, int32_t k, int32_t xtype, cudaStream_t s,
+                                 cudaError_t* e, int32_t* chunk);
 struct FwdArgs;
 // Lane geometry of one call: VEC elements per lane load (the widest vector
 // that divides k and keeps every X load and Y store aligned), CH column
@@ -350,12 +350,18 @@ struct FwdArgs {
     // short-row runs over rows of several lanes: 1 = merge-based pieces per
     // lane group, 0 = each group walks whole rows
     int32_t merge_groups = 0;
+    int32_t x_large = 0;   // X takes more than kLargeXBytes
     // hot variant: a negative column index c names row ~c of the hot rows,
     // hot_bytes (a multiple of 16) of them packed at Xh, copied into shared
     // memory at the start of each block
     const void* Xh = nullptr;
     int64_t hot_bytes = 0;
 };
+
+// X beyond the part of L2 that random gathers fill (64 MB of the GPU's L2: uniform
+// gathers of 32-byte rows run at 304 G rows/s from a 64 MB table, 125 from
+// 128 MB, 76 from 256 MB).
+constexpr int64_t kLargeXBytes = 64ll << 20;
 
 // One launch over the tasks of several matrices (spmm_apply_batched): the
 // entries' arguments travel in the kernel's parameter space (no device
@@ -385,6 +391,18 @@ constexpr int kWideRowBytes = 16;
 #define SPMM_NARROW_TASK_CHUNK 8
 #endif
 constexpr int kNarrowTaskChunk = SPMM_NARROW_TASK_CHUNK;
+// Short lists are claimed fewer at a time: a launch has about 3,600 warps, and
+// with eight tasks per claim a list of 5,000 left most of them idle while 170
+// worked through nine tasks each (R-MAT, k = 1: 64 K vertices, 5,002 tasks
+// 27.2 -> 16.6 us; 512 K, 36,046 tasks 46.5 -> 39.3 us).  One more per claim for
+// every 16,384 tasks (four and a half per warp) reaches the eight of long lists at 131,072.
+constexpr int64_t kTasksPerChunk = 16384;
+inline int32_t claim_chunk(int64_t n_tasks, bool wide) {
+    const int64_t c = n_tasks / kTasksPerChunk;
+    return wide || c < 1 ? 1 : c > kNarrowTaskChunk ? kNarrowTaskChunk : (int32_t)c;
+}
+// most tasks of one launch (the kernel numbers them in 32 bits)
+constexpr int64_t kMaxLaunchTasks = 1ll << 31;
 
 // rows_*.cu: launch the task kernel for one X dtype.  vmode: 0 pattern,
 // 1 f32 values, 2 bf16 values, 3 f16 values.  Returns a cudaError_t.

@@ -6,6 +6,7 @@
 namespace spmm {
 
 cudaError_t launch_rows_bf16_mg(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s) {
+    if (vmode != 0 && (vec < 4 || a.x_large)) return launch_rows_t<__nv_bfloat16, false, 3>(a, vmode, vec, ch, s);
     return launch_rows_t<__nv_bfloat16, false, 1>(a, vmode, vec, ch, s);
 }
 

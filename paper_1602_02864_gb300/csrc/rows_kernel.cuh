@@ -251,21 +251,27 @@ struct Layout {
 struct Staged {
     const int32_t* col;         // col[i] = column of nonzero e0 + i
     const unsigned char* val;   // raw value bytes, entry i = nonzero e0 + i
-    const int64_t* rp;          // rp[j] = row_ptr[r0 + j] (short-row tasks)
+    const int64_t* rpw;         // staged row_ptr[r0 ..] (short-row tasks)
+    int e0;                     // low word of the task's first nonzero
+    // start of row j among the task's nonzeros (the low words' difference)
+    __device__ __forceinline__ int rp(int j) const {
+        return (int)(reinterpret_cast<const uint32_t*>(rpw)[2 * j] - (uint32_t)e0);
+    }
 };
 
-__device__ __forceinline__ int64_t desc_e0(const int4 d) {
-    return ((int64_t)(uint32_t)d.z) | ((int64_t)d.w << 32);
+__device__ __forceinline__ int64_t desc_e0(int z, int w) {
+    return ((int64_t)(uint32_t)z) | ((int64_t)w << 32);
 }
 
 // Issue the bulk copies of one task into staging buffer `buf` (lane 0 only).
 // Windows are widened to 16-byte boundaries; the arrays are padded on the
 // device so the widened end stays inside the allocation.
 template <int VMODE>
-__device__ __forceinline__ void issue_task(const FwdArgs& a, const int4 d0, const int4 d1, unsigned char* buf,
-                                           uint64_t* bar, uint64_t pol) {
+__device__ __forceinline__ void issue_task(const FwdArgs& a, const int4 d0, int64_t e1, unsigned char* buf,
+                                           uint64_t* bar) {
     using Lay = Layout<VMODE>;
-    const int64_t e0 = desc_e0(d0), e1 = desc_e0(d1);
+    const uint64_t pol = policy_evict_first();
+    const int64_t e0 = desc_e0(d0.z, d0.w);
     const int64_t cs = e0 & ~(int64_t)3, ce = (e1 + 3) & ~(int64_t)3;
     const uint32_t cbytes = (uint32_t)((ce - cs) * 4);
     uint32_t vbytes = 0, rbytes = 0;
@@ -313,17 +319,33 @@ __device__ __forceinline__ void issue_task(const FwdArgs& a, const int4 d0, cons
 // (R-MAT scale 24, FP32: k = 1 1.10 -> 0.93 ms, k = 8 2.23 -> 1.92, 30
 // PageRank iterations 35.9 -> 31.6 ms; k = 32 4.20 -> 4.34, k = 64
 // 7.59 -> 7.91), which keeps four in its own variant (MG == 2).
-template <int VMODE, int MG>
+// Two blocks, with twice the gathers in flight (up to 128 registers): where the
+// staged values double the staging buffers, three blocks take 226 KB of
+// shared memory and leave L1 next to nothing (weighted R-MAT, 4 M vertices,
+// FP32, ms with three -> two: k = 1 0.395 -> 0.252, k = 2 0.424 -> 0.291, k = 8
+// 0.684 -> 0.440; BF16 X, k = 16 0.771 -> 0.622; 2 M, k = 64 1.081 -> 0.834), and
+// for rows on two chunks of single elements (FP16, k = 33, 700 K vertices
+// 0.492 -> 0.443).  Pattern rows on one chunk lose (k = 8, 8 M vertices 0.90 ->
+// 1.03 ms, k = 32, 4 M 1.03 -> 1.19).  The weighted group merge comes in both
+// forms (MG == 1, MG == 3): lanes of 16 bytes run faster with three blocks while X
+// fits L2 (k = 16, 37 MB of X: 0.152 against 0.162 ms) and with two beyond
+// (134 MB: 0.836 against 0.569), narrower lanes always with two (k = 4, 67 MB
+// 0.510 against 0.433).
+template <int VMODE, int CH, bool ONE, int MG>
+constexpr bool two_blocks() {
+    return (VMODE != 0 && MG == 0) || MG == 3 || CH == 2;
+}
+template <int VMODE, int CH, bool ONE, int MG>
 constexpr int min_blocks() {
-    return (MG == 2 && VMODE == 0) ? 4 : SPMM_MIN_BLOCKS;
+    return (MG == 2 && VMODE == 0) ? 4 : two_blocks<VMODE, CH, ONE, MG>() ? 2 : SPMM_MIN_BLOCKS;
 }
 
 // ONE: one lane per X row (k == VEC, CH == 1); the lane geometry is then a
 // compile-time constant and short-row runs take the flat (k = 1) or, for X
 // rows of up to 8 bytes, the merge-based path.  MG != 0: several lanes per X
 // row (CH == 1) and short-row runs merge-based over lane groups, with 3
-// blocks per SM and 4 nonzeros in flight per group (MG == 1) or 4 blocks and
-// 2 in flight (MG == 2).
+// blocks per SM and 4 nonzeros in flight per group (MG == 1), 4 blocks and 2 in
+// flight (MG == 2) or 2 blocks and 8 in flight (MG == 3).
 // Warps per block: kWarpsPerBlock, or kHotWarps in one block per SM for the
 // instantiations that keep the hot rows of X in shared memory (HOT).
 template <bool HOT>
@@ -355,7 +377,8 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     using Lay = Layout<VMODE>;
     // nonzeros in flight per lane group
     constexpr int kBytes = VEC * CH * (int)sizeof(XT);
-    constexpr int kU = SPMM_UNROLL_BYTES / kBytes;
+    constexpr bool kWide = MULTI || (two_blocks<VMODE, CH, ONE, MG>() && !HOT);
+    constexpr int kU = SPMM_UNROLL_BYTES * (kWide ? 2 : 1) / kBytes;
     constexpr int U = kU < 2 ? 2 : (kU > 8 ? 8 : kU);
 #ifndef SPMM_MERGE_UNROLL
 #define SPMM_MERGE_UNROLL 2
@@ -364,9 +387,11 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
 #ifndef SPMM_MERGE_WIDE_UNROLL
 #define SPMM_MERGE_WIDE_UNROLL 4
 #endif
-    // merge over lane groups: nonzeros in flight per group (4 spill at 64
-    // registers, and with staged values at 80)
-    constexpr int kUW = (MG == 1 && VMODE == 0) ? SPMM_MERGE_WIDE_UNROLL : 2;
+    // merge over lane groups: nonzeros in flight per group.  Values are read from
+    // shared memory when they are used and the task state fits few registers, so
+    // 4 in flight spill neither with values (2 before: k = 16 weighted, 37 MB of
+    // X 0.168 -> 0.152 ms) nor without; 6 do (0.211).
+    constexpr int kUW = MG == 3 ? 2 * SPMM_MERGE_WIDE_UNROLL : MG == 1 ? SPMM_MERGE_WIDE_UNROLL : 2;
     constexpr int UW = U < kUW ? U : kUW;
     extern __shared__ __align__(128) unsigned char smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -395,9 +420,10 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
         }
     }
 
-    const int64_t W = (int64_t)gridDim.x * WPB;
-    int64_t t = (int64_t)blockIdx.x * WPB + w;
-    if (t >= a.n_tasks) return;
+    const uint32_t n_tasks = (uint32_t)a.n_tasks;      // at most kMaxLaunchTasks
+    const uint32_t W = gridDim.x * WPB;
+    const uint32_t t = blockIdx.x * WPB + w;
+    if (t >= n_tasks) return;
     if (lane == 0) {
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
@@ -405,23 +431,28 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     }
     __syncwarp();
 
-    // the entry of task t (MULTI: a binary search of the entries' first tasks)
-    // and its two descriptors
-    auto fetch = [&](int64_t tt, int4& x0, int4& x1) -> int {
+    // a task's descriptor and where it ends (the next one's first nonzero)
+    struct Desc {
+        int4 a;
+        int2 end;
+    };
+    auto load_desc = [&](const int4* p, Desc& x) {
+        x.a = p[0];
+        x.end = reinterpret_cast<const int2*>(p + 1)[1];
+    };
+    // returns the task's entry (MULTI: a binary search of the entries' first tasks)
+    auto fetch = [&](uint32_t tt, Desc& x) -> int {
         if constexpr (MULTI) {
             int lo = 0, hi = M->n - 1;
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
-                if (M->off[mid] <= tt) lo = mid;
+                if (M->off[mid] <= (int64_t)tt) lo = mid;
                 else hi = mid - 1;
             }
-            const int64_t tl = tt - M->off[lo];
-            x0 = M->ent[lo].tasks[tl];
-            x1 = M->ent[lo].tasks[tl + 1];
+            load_desc(M->ent[lo].tasks + ((int64_t)tt - M->off[lo]), x);
             return lo;
         } else {
-            x0 = a.tasks[tt];
-            x1 = a.tasks[tt + 1];
+            load_desc(a.tasks + tt, x);
             return 0;
         }
     };
@@ -434,7 +465,6 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     int lg = 0, LANES = 1, G = 32, g = 0, li = 0;
     bool act[CH];
     const XT* xb = nullptr;
-    const uint64_t apol = policy_evict_first();
     uint64_t xpol = 0;
     const FwdArgs* cur = &a;    // the entry of the task being computed
     auto set_geometry = [&](const FwdArgs& E) {
@@ -457,49 +487,61 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                 return;
             }
         }
-        xv.load(xb + c * cur->ldx + off, xpol);
+        xv.load(xb + (uint64_t)(uint32_t)c * (uint64_t)cur->ldx + off, xpol);
     };
-    int4 d0, d1;
-    int ed = fetch(t, d0, d1);
+    // copy the task in x (fetch) into buffer buf (lane 0 issues)
+    auto stage = [&](int e, const Desc& x, int buf) {
+        if (lane == 0)
+            issue_task<VMODE>(entry(e), x.a, desc_e0(x.end.x, x.end.y), wb + buf * Lay::kBuf, &bars[buf]);
+    };
+    Desc nx;
+    int ed = fetch(t, nx);
     set_geometry(entry(ed));
-    if (lane == 0) issue_task<VMODE>(entry(ed), d0, d1, wb, &bars[0], apol);
+    stage(ed, nx, 0);
+    // the current task: first row, kind, low word of its first nonzero, nonzeros
+    int2 d0;
+    int e0, n;
+    auto take = [&](const Desc& x) {
+        d0 = make_int2(x.a.x, x.a.y);
+        e0 = x.a.z;
+        n = x.end.x - e0;
+    };
+    take(nx);
     // the next task: static stride, or the next of a chunk claimed from the
     // counter by lane 0
-    int64_t cnext = 0, cend = 0;
-    auto next_task = [&](int64_t cur) -> int64_t {
+    uint32_t cnext = 0, cend = 0;
+    auto next_task = [&](uint32_t cur) -> uint32_t {
         if (!a.task_ctr) return cur + W;
         if (cnext < cend) return cnext++;
-        unsigned long long v = 0;
-        if (lane == 0) v = atomicAdd(a.task_ctr, 1ull);
-        cnext = W + (int64_t)__shfl_sync(0xffffffffu, v, 0) * a.task_chunk;
+        uint32_t v = 0;
+        if (lane == 0) v = atomicAdd(reinterpret_cast<unsigned int*>(a.task_ctr), 1u);
+        cnext = W + __shfl_sync(0xffffffffu, v, 0) * (uint32_t)a.task_chunk;
         cend = cnext + a.task_chunk;
         return cnext++;
     };
-    int64_t tn = next_task(t);
-    int4 n0 = make_int4(0, 0, 0, 0), n1 = n0;
+    uint32_t tn = next_task(t);
     int en = 0;
-    if (tn < a.n_tasks) en = fetch(tn, n0, n1);
+    if (tn < n_tasks) en = fetch(tn, nx);
     uint32_t phase = 0;     // bit b = parity to wait for on buffer b
     int b = 0;
 
     for (;;) {
         // stage the next task into the other buffer (its readers are done)
-        if (tn < a.n_tasks) {
+        const bool more = tn < n_tasks;
+        if (more) {
             __syncwarp();
-            if (lane == 0) {
-                fence_proxy_async();
-                issue_task<VMODE>(entry(en), n0, n1, wb + (b ^ 1) * Lay::kBuf, &bars[b ^ 1], apol);
-            }
+            if (lane == 0) fence_proxy_async();
+            stage(en, nx, b ^ 1);
         }
         // prefetch the descriptor after next
-        const int64_t tnn = tn < a.n_tasks ? next_task(tn) : a.n_tasks;
-        int4 m0 = make_int4(0, 0, 0, 0), m1 = m0;
+        const uint32_t tnn = more ? next_task(tn) : n_tasks;
+        Desc mx{};
         int em = 0;
-        if (tnn < a.n_tasks) em = fetch(tnn, m0, m1);
+        if (tnn < n_tasks) em = fetch(tnn, mx);
 
         if (!mbar_wait_bounded(&bars[b], (phase >> b) & 1u, a.wait_ns)) {
             if (lane == 0) atomicOr(a.status, kStatusTimeout);
-            if (tn < a.n_tasks) mbar_wait_bounded(&bars[b ^ 1], (phase >> (b ^ 1)) & 1u, a.wait_ns);
+            if (more) mbar_wait_bounded(&bars[b ^ 1], (phase >> (b ^ 1)) & 1u, a.wait_ns);
             return;
         }
         phase ^= 1u << b;
@@ -511,9 +553,8 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
         {
             const FwdArgs& a = *cur;   // the task's entry (the launch's matrix unless MULTI)
             const unsigned char* buf = wb + b * Lay::kBuf;
-            const int64_t e0 = desc_e0(d0);
-            const int n = (int)(desc_e0(d1) - e0);
             Staged st;
+            st.e0 = e0;
             st.col = reinterpret_cast<const int32_t*>(buf + Lay::kColOff) + (e0 & 3);
             if constexpr (VMODE != 0) {
                 constexpr int epb = 16 / Lay::kValBytes;
@@ -521,7 +562,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
             } else {
                 st.val = nullptr;
             }
-            st.rp = reinterpret_cast<const int64_t*>(buf + Lay::kRpOff) + (d0.x & 1);
+            st.rpw = reinterpret_cast<const int64_t*>(buf + Lay::kRpOff) + (d0.x & 1);
 
             if (kFlat && d0.y > 0) {
                 // k = 1, run of short rows: every lane gathers the task's
@@ -552,7 +593,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                 }
                 __syncwarp();
                 for (int j = lane; j < nr; j += 32) {
-                    const int s = (int)(st.rp[j] - e0), e = (int)(st.rp[j + 1] - e0);
+                    const int s = st.rp(j), e = st.rp(j + 1);
                     float acc = 0.f;
                     for (int i = s; i < e; i += 4) {          // four loads in flight, added in order
                         const float p0 = __int_as_float(prod[i]);
@@ -579,7 +620,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                 // adds the tails, and the ending lane adds its head last.
                 const int nr = d0.y;
                 for (int j = lane; j < nr; j += 32)       // rows without nonzeros
-                    if (st.rp[j] == st.rp[j + 1]) {
+                    if (st.rp(j) == st.rp(j + 1)) {
                         float z[VEC];
 #pragma unroll
                         for (int v = 0; v < VEC; ++v) z[v] = 0.f;
@@ -597,11 +638,11 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                     int lo = 0, hi = nr - 1;
                     while (lo < hi) {
                         const int mid = (lo + hi + 1) >> 1;
-                        if ((int)(st.rp[mid] - e0) <= cs) lo = mid;
+                        if (st.rp(mid) <= cs) lo = mid;
                         else hi = mid - 1;
                     }
                     int r = lo;
-                    int rs = (int)(st.rp[r] - e0), re = (int)(st.rp[r + 1] - e0);
+                    int rs = st.rp(r), re = st.rp(r + 1);
                     float acc[VEC];
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) acc[v] = 0.f;
@@ -632,7 +673,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                                     for (int v = 0; v < VEC; ++v) acc[v] = 0.f;
                                     ++r;
                                     rs = re;
-                                    re = (int)(st.rp[r + 1] - e0);
+                                    re = st.rp(r + 1);
                                 }
 #pragma unroll
                                 for (int v = 0; v < VEC; ++v) acc[v] = fmaf(av[u], xv[u].get(v), acc[v]);
@@ -679,7 +720,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                 // li of a group meets lane li of the others) and its head.
                 const int nr = d0.y;
                 for (int j = g; j < nr; j += G)           // rows without nonzeros
-                    if (st.rp[j] == st.rp[j + 1] && act[0]) {
+                    if (st.rp(j) == st.rp(j + 1) && act[0]) {
                         float z[VEC];
 #pragma unroll
                         for (int v = 0; v < VEC; ++v) z[v] = 0.f;
@@ -696,22 +737,20 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                     int lo = 0, hi = nr - 1;              // the row holding nonzero cs
                     while (lo < hi) {
                         const int mid = (lo + hi + 1) >> 1;
-                        if ((int)(st.rp[mid] - e0) <= cs) lo = mid;
+                        if (st.rp(mid) <= cs) lo = mid;
                         else hi = mid - 1;
                     }
                     int r = lo;
-                    int rs = (int)(st.rp[r] - e0), re = (int)(st.rp[r + 1] - e0);
+                    int rs = st.rp(r), re = st.rp(r + 1);
                     float acc[VEC];
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) acc[v] = 0.f;
                     for (int i = cs; i < ce; i += UW) {
                         XVec<XT, VEC> xv[UW];
-                        float av[UW];
 #pragma unroll
                         for (int u = 0; u < UW; ++u)
                             if (i + u < ce) {
                                 const int64_t cidx = st.col[i + u];
-                                av[u] = staged_val<VMODE>(st.val, i + u);
                                 if (act[0]) gather(xv[u], cidx, 0);
                             }
 #pragma unroll
@@ -731,11 +770,12 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                                     for (int v = 0; v < VEC; ++v) acc[v] = 0.f;
                                     ++r;
                                     rs = re;
-                                    re = (int)(st.rp[r + 1] - e0);
+                                    re = st.rp(r + 1);
                                 }
                                 if (act[0]) {
+                                    const float av = staged_val<VMODE>(st.val, i + u);
 #pragma unroll
-                                    for (int v = 0; v < VEC; ++v) acc[v] = fmaf(av[u], xv[u].get(v), acc[v]);
+                                    for (int v = 0; v < VEC; ++v) acc[v] = fmaf(av, xv[u].get(v), acc[v]);
                                 }
                             }
                     }
@@ -767,7 +807,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                 // run of short rows: lane group g owns rows g, g+G, ...
                 const int nr = d0.y;
                 for (int j = g; j < nr; j += G) {
-                    const int s = (int)(st.rp[j] - e0), e = (int)(st.rp[j + 1] - e0);
+                    const int s = st.rp(j), e = st.rp(j + 1);
                     float acc[CH][VEC];
 #pragma unroll
                     for (int c = 0; c < CH; ++c)
@@ -775,12 +815,10 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                         for (int v = 0; v < VEC; ++v) acc[c][v] = 0.f;
                     for (int i = s; i < e; i += U) {
                         XVec<XT, VEC> xv[U][CH];
-                        float av[U];
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             if (i + u < e) {
                                 const int64_t cidx = st.col[i + u];
-                                av[u] = staged_val<VMODE>(st.val, i + u);
 #pragma unroll
                                 for (int c = 0; c < CH; ++c)
                                     if (act[c]) gather(xv[u][c], cidx, c * LANES * VEC);
@@ -789,10 +827,11 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
 #pragma unroll
                         for (int u = 0; u < U; ++u)
                             if (i + u < e) {
+                                const float av = staged_val<VMODE>(st.val, i + u);
 #pragma unroll
                                 for (int c = 0; c < CH; ++c)
 #pragma unroll
-                                    for (int v = 0; v < VEC; ++v) acc[c][v] = fmaf(av[u], xv[u][c].get(v), acc[c][v]);
+                                    for (int v = 0; v < VEC; ++v) acc[c][v] = fmaf(av, xv[u][c].get(v), acc[c][v]);
                             }
                     }
                     float* dst = a.Y + (int64_t)(d0.x + j) * a.ldy;
@@ -884,13 +923,11 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                     for (int v = 0; v < VEC; ++v) acc[c][v] = 0.f;
                 for (int i = g; i < n; i += G * U) {
                     XVec<XT, VEC> xv[U][CH];
-                    float av[U];
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         const int idx = i + u * G;
                         if (idx < n) {
                             const int64_t cidx = st.col[idx];
-                            av[u] = staged_val<VMODE>(st.val, idx);
 #pragma unroll
                             for (int c = 0; c < CH; ++c)
                                 if (act[c]) gather(xv[u][c], cidx, c * LANES * VEC);
@@ -899,10 +936,11 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
 #pragma unroll
                     for (int u = 0; u < U; ++u)
                         if (i + u * G < n) {
+                            const float av = staged_val<VMODE>(st.val, i + u * G);
 #pragma unroll
                             for (int c = 0; c < CH; ++c)
 #pragma unroll
-                                for (int v = 0; v < VEC; ++v) acc[c][v] = fmaf(av[u], xv[u][c].get(v), acc[c][v]);
+                                for (int v = 0; v < VEC; ++v) acc[c][v] = fmaf(av, xv[u][c].get(v), acc[c][v]);
                         }
                 }
                 for (int off = LANES; off < 32; off <<= 1)
@@ -921,16 +959,18 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                 }
             }
         }
-        if (tn >= a.n_tasks) break;
-        d0 = n0; d1 = n1; ed = en;
-        n0 = m0; n1 = m1; en = em;
+        if (!more) break;
+        take(nx);
+        ed = en;
+        nx = mx;
+        en = em;
         tn = tnn;
         b ^= 1;
     }
 }
 
 template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG = 0, bool HOT = false>
-__global__ void __launch_bounds__(warps_per_block<HOT>() * 32, (HOT ? 1 : min_blocks<VMODE, MG>()))
+__global__ void __launch_bounds__(warps_per_block<HOT>() * 32, (HOT ? 1 : min_blocks<VMODE, CH, ONE, MG>()))
     rows_kernel(const __grid_constant__ FwdArgs a) {
     rows_run<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT, false>(a, nullptr);
 }
@@ -1065,6 +1105,14 @@ cudaError_t launch_rows_t(const FwdArgs& a, int vmode, int vec, int ch, cudaStre
                              : launch_one<XT, VM, V, C, false, ONE, MG>(a, s);
     if constexpr (MG == 2) {     // float pattern rows of 4-element lanes only
         if constexpr (sizeof(XT) == 4) { SPMM_LAUNCH(0, 4, 1) }
+    } else if constexpr (MG == 3) {   // staged values only
+        if constexpr (sizeof(XT) == 4) {
+            SPMM_LAUNCH(1, 4, 1) SPMM_LAUNCH(1, 2, 1) SPMM_LAUNCH(1, 1, 1)
+        } else {
+            constexpr int VM3 = std::is_same<XT, __half>::value ? 3 : 2;
+            SPMM_LAUNCH(1, 4, 1) SPMM_LAUNCH(1, 2, 1) SPMM_LAUNCH(1, 1, 1)
+            SPMM_LAUNCH(VM3, 4, 1) SPMM_LAUNCH(VM3, 2, 1) SPMM_LAUNCH(VM3, 1, 1)
+        }
     } else if constexpr (MG == 1) {   // CH == 1, at most 4 elements per lane
         if constexpr (sizeof(XT) == 4) {
             SPMM_LAUNCH(0, 4, 1) SPMM_LAUNCH(0, 2, 1) SPMM_LAUNCH(0, 1, 1)

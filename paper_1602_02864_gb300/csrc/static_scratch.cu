@@ -161,9 +161,7 @@ extern "C" int spmm_apply_csr_static(int64_t n_rows, int64_t n_cols, int64_t nnz
     a.compensated = 0;
     a.partials_comp = nullptr;
     const int vec = gm.vec, ch = gm.ch;
-    if (xtype == SPMM_F32) e = launch_rows_f32(a, vmode, vec, ch, s);
-    else if (xtype == SPMM_BF16) e = launch_rows_bf16(a, vmode, vec, ch, s);
-    else e = launch_rows_f16(a, vmode, vec, ch, s);
+    e = launch_rows(a, (int32_t)xtype, vmode, vec, ch, s);
     if (e != cudaSuccess) {
         set_error(std::string("spmm_apply_csr_static: task kernel: ") + cudaGetErrorString(e));
         return SPMM_ERR_CUDA;

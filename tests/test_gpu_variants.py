@@ -1,0 +1,63 @@
+"""Variants of the task kernel that are chosen by size: the weighted merge over
+lane groups with two or three blocks per SM, and the tasks claimed at a time."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sp():
+    from paper_1602_02864_gb300 import spmm
+    return spmm
+
+
+@pytest.mark.parametrize("xdtype", ["float32", "bfloat16", "float16"])
+@pytest.mark.parametrize("k", [2, 4, 6, 12, 16, 32])
+def test_large_x_variant_same_sums(sp, xdtype, k):
+    """A row stride that makes X count as larger than L2 takes the two-block form:
+    the same pieces and sums, so the same bits as the three-block form on a dense X, and
+    both match the oracle."""
+    import torch
+    A = synth.rmat_csr(14, seed=5, weighted=True)
+    h = sp.SparseMatrix.from_csr(A, transpose=True, opts=sp.spmm_opts(short_runs=2))
+    try:
+        n, dt = A.n_rows, getattr(torch, xdtype)
+        X = torch.from_numpy(synth.dense(n, k, seed=k)).cuda().to(dt)
+        wide = torch.zeros((n, 1536 if xdtype == "float32" else 3072), dtype=dt, device="cuda")
+        assert wide.numel() * wide.element_size() > 64 << 20
+        wide[:, :k] = X
+        Xh = X.float().cpu().numpy()
+        for tr in (False, True):
+            Y, Yw = h.apply(X, transpose=tr), h.apply(wide[:, :k], transpose=tr)
+            assert torch.equal(Y, Yw)
+            ref = oracle.spmm(n, n, A.row_ptr, A.col_idx, A.values, Xh, transpose=tr)
+            scale = oracle.spmm(n, n, A.row_ptr, A.col_idx, A.values, np.abs(Xh), transpose=tr)
+            assert np.all(np.abs(Y.cpu().numpy() - ref) <= 1e-5 * scale + 1e-30)
+    finally:
+        h.close()
+
+
+@pytest.mark.parametrize("n_tasks", [1, 4000, 16383, 16384, 32768, 60000, 131072, 140000])
+@pytest.mark.parametrize("k", [1, 2])
+def test_every_task_claimed_once(sp, n_tasks, k):
+    """Lists of as many one-row tasks as make the claim size change (1 to 8 at a time):
+    every row is written, with its exact sum."""
+    import torch
+    rng = np.random.default_rng(n_tasks)
+    deg = rng.integers(0, 5, n_tasks)
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int64)
+    cols = rng.integers(0, 1000, rp[-1]).astype(np.int32)
+    h = sp.SparseMatrix(n_tasks, 1000, rp, cols, None, opts=sp.spmm_opts(task_rows=1))
+    try:
+        assert h.info()["n_tasks"] == n_tasks
+        X = synth.dense(1000, k, seed=1, mode="int")
+        Y = torch.full((n_tasks, k), -1.0, device="cuda")
+        h.apply(torch.from_numpy(X).cuda(), Y=Y)
+        ref = oracle.spmm(n_tasks, 1000, rp, cols, None, X)
+        assert np.array_equal(Y.cpu().numpy().astype(np.float64), ref)
+    finally:
+        h.close()
