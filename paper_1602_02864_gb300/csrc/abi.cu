@@ -52,10 +52,11 @@ static void free_dev(DevCSR& d) {
     cudaFree(d.partials);
     cudaFree(d.partials_comp);
     cudaFree(d.perm);
-    cudaFree(d.task_ctr);
+    cudaFree(d.ctl);
+    cudaFree(d.slot_seg);
+    cudaFree(d.seg_done);
     cudaFree(d.col_hot);
     cudaFree(d.hot_cols);
-    cudaFree(d.xh);
     d = DevCSR{};
 }
 
@@ -71,6 +72,19 @@ static cudaError_t upload(T** dst, const T* src, size_t count, size_t pad, cudaS
     if (pad && (e = cudaMemsetAsync(*dst + count, 0, pad * sizeof(T), s)) != cudaSuccess) return e;
     if (count == 0) return cudaSuccess;
     return cudaMemcpyAsync(*dst, src, count * sizeof(T), cudaMemcpyHostToDevice, s);
+}
+
+// The split and segments of each partial slot's row and the (zero) arrivals at
+// each split row, on the device.
+static cudaError_t upload_split_state(const HostPlan& plan, int2** slot_seg, unsigned int** seg_done, cudaStream_t s,
+                                      int64_t* bytes) {
+    std::vector<int2> of((size_t)plan.n_slots);
+    for (size_t i = 0; i < plan.splits.size(); ++i)
+        std::fill_n(of.begin() + plan.splits[i].z, plan.splits[i].y, make_int2((int)i, plan.splits[i].y));
+    cudaError_t e = upload(slot_seg, of.data(), of.size(), 0, s, bytes);
+    if (e == cudaSuccess) e = upload(seg_done, (const unsigned int*)nullptr, 0, plan.splits.size(), s, bytes);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);    // `of` is freed on return
+    return e;
 }
 
 // Copy one orientation (host CSR) and its plan to the device.
@@ -116,12 +130,6 @@ static int build_orientation(DevCSR& d, int64_t n_rows, int64_t n_cols, const in
         if ((e = upload(&d.col_hot, encoded.data(), (size_t)d.nnz, 8, s, bytes)) != cudaSuccess ||
             (e = upload(&d.hot_cols, hot.data(), hot.size(), 0, s, bytes)) != cudaSuccess)
             return cuda_fail(e, "hot columns");
-        const size_t xb = (hot.size() * kHotRowBytes + 15) & ~(size_t)15;
-        if ((e = cudaMalloc(&d.xh, xb)) != cudaSuccess) {
-            d.xh = nullptr;
-            return cuda_fail(e, "hot rows of X");
-        }
-        *bytes += (int64_t)xb;
         d.n_hot = (int64_t)hot.size();
     }
     // the host vectors are freed on return: finish their copies first
@@ -138,11 +146,10 @@ static int build_orientation(DevCSR& d, int64_t n_rows, int64_t n_cols, const in
     d.n_splits = (int64_t)plan.splits.size();
     d.n_segments = plan.n_segments;
     d.n_slots = plan.n_slots;
-    if ((e = cudaMalloc((void**)&d.task_ctr, sizeof(unsigned long long))) != cudaSuccess) {
-        d.task_ctr = nullptr;
-        return cuda_fail(e, "task counter");
-    }
-    *bytes += (int64_t)sizeof(unsigned long long);
+    const TaskCtl zero{};
+    if ((e = upload(&d.ctl, &zero, 1, 0, s, bytes)) != cudaSuccess) return cuda_fail(e, "task counter");
+    if ((e = upload_split_state(plan, &d.slot_seg, &d.seg_done, s, bytes)) != cudaSuccess)
+        return cuda_fail(e, "split rows");
     if (d.n_slots > 0) {
         size_t pb = (size_t)d.n_slots * kSlotStride * sizeof(float);
         if ((e = cudaMalloc((void**)&d.partials, pb)) != cudaSuccess) { d.partials = nullptr; return cuda_fail(e, "partials"); }
@@ -656,14 +663,8 @@ extern "C" int spmm_create_batched(spmm_mat_t* out, int32_t n_graphs, const int6
 
 namespace spmm {
 
-// The task counter of a launch (reset on s) and the tasks claimed at a time.
-unsigned long long* task_counter(const DevCSR& d, int64_t n_tasks, int32_t k, int32_t xtype, cudaStream_t s,
-                                 cudaError_t* e, int32_t* chunk) {
-    *e = cudaSuccess;
-    *chunk = claim_chunk(n_tasks, (int64_t)k * (int64_t)dtype_size((spmm_dtype)xtype) >= kWideRowBytes);
-    if (!d.task_ctr) return nullptr;
-    *e = cudaMemsetAsync(d.task_ctr, 0, sizeof(unsigned long long), s);
-    return *e == cudaSuccess ? d.task_ctr : nullptr;
+int32_t task_chunk_of(int64_t n_tasks, int32_t k, int32_t xtype) {
+    return claim_chunk(n_tasks, (int64_t)k * (int64_t)dtype_size((spmm_dtype)xtype) >= kWideRowBytes);
 }
 
 LaneGeometry lane_geometry(const void* X, int64_t ldx, int32_t k, int32_t xtype, const float* Y, int64_t ldy) {
@@ -735,7 +736,7 @@ cudaError_t launch_rows(const FwdArgs& all, int32_t xtype, int vmode, int vec, i
         FwdArgs a = all;
         a.tasks = all.tasks + t0;
         a.n_tasks = std::min(kMaxLaunchTasks, all.n_tasks - t0);
-        if (t0 > 0) a.task_ctr = nullptr;
+        if (t0 > 0) a.task_chunk = 0;
         if (xtype == SPMM_F32) e = launch_rows_f32(a, vmode, vec, ch, s);
         else if (xtype == SPMM_BF16) e = launch_rows_bf16(a, vmode, vec, ch, s);
         else e = launch_rows_f16(a, vmode, vec, ch, s);
@@ -767,13 +768,11 @@ static int apply_resident(const spmm_mat* A, int transpose, const void* X, int64
     const int esize = (int)dtype_size(xtype);
     a.col_idx = d.col_idx;
     if (d.n_hot > 0 && k * esize == kHotRowBytes && ch == 1 && a.lanes_log2 == 0) {
-        // one lane per 4-byte X row: the hot variant, fed with the packed hot
-        // rows of X and the column indices that name them
-        const cudaError_t eh = hot_gather(d, X, ldx, k, esize, s);
-        if (eh != cudaSuccess) return cuda_fail(eh, "spmm_apply: hot rows");
+        // one lane per 4-byte X row: the hot variant, with the column indices that
+        // name the hot rows
         a.col_idx = d.col_hot;
-        a.Xh = d.xh;
-        a.hot_bytes = (d.n_hot * k * esize + 15) & ~(int64_t)15;
+        a.hot_cols = d.hot_cols;
+        a.n_hot = d.n_hot;
     }
     a.row_ptr = d.row_ptr;
     a.val = d.val;
@@ -784,20 +783,28 @@ static int apply_resident(const spmm_mat* A, int transpose, const void* X, int64
     a.x_evict_last = A->params.x_evict_last;
     a.compensated = d.partials_comp != nullptr || (A->params.compensated && d.n_slots == 0);
     a.partials_comp = d.partials_comp;
+    a.ctl = d.ctl;
+    const bool combine_inside = combines_inside(d) && !a.compensated && !a.hot_cols;
+    if (combine_inside) {         // a run holds all segments of its split rows
+        a.splits = d.splits;
+        a.n_splits = d.n_splits;
+        a.slot_seg = d.slot_seg;
+        a.seg_done = d.seg_done;
+    }
     const RowBlock all{0, d.n_tasks, 0, d.n_rows, 0, d.n_splits};
     const bool by_runs = rows_done && d.row_blocks.size() > 1;
     const size_t n_runs = by_runs ? d.row_blocks.size() : 1;
     for (size_t j = 0; j < n_runs; ++j) {
         const RowBlock& b = by_runs ? d.row_blocks[j] : all;
-        cudaError_t ec = cudaSuccess;
-        a.task_ctr = task_counter(d, b.t1 - b.t0, k, xtype, s, &ec, &a.task_chunk);
-        if (ec != cudaSuccess) return cuda_fail(ec, "spmm_apply: task counter");
+        a.task_chunk = task_chunk_of(b.t1 - b.t0, k, xtype);
         a.tasks = d.tasks + b.t0;
         a.n_tasks = b.t1 - b.t0;
         cudaError_t e = launch_rows(a, xtype, vmode, vec, ch, s);
         if (e != cudaSuccess) return cuda_fail(e, "spmm_apply: task kernel");
-        e = launch_combine(d.splits + b.s0, b.s1 - b.s0, d.partials, Y, ldy, k, s, d.partials_comp);
-        if (e != cudaSuccess) return cuda_fail(e, "spmm_apply: combine kernel");
+        if (!combine_inside) {
+            e = launch_combine(d.splits + b.s0, b.s1 - b.s0, d.partials, Y, ldy, k, s, d.partials_comp);
+            if (e != cudaSuccess) return cuda_fail(e, "spmm_apply: combine kernel");
+        }
         if (rows_done) {
             const int rc = (*rows_done)(b.r0, b.r1);
             if (rc != SPMM_OK) return rc;
@@ -977,25 +984,35 @@ static int replan_orientation(DevCSR& d, const Params& p, cudaStream_t s, int64_
     HostPlan plan = build_plan(rp.data(), d.n_rows, p);
     int4 *tasks = nullptr, *splits = nullptr;
     float *partials = nullptr, *pcomp = nullptr;
+    int2* slot_seg = nullptr;
+    unsigned int* seg_done = nullptr;
     int64_t added = 0;
     const size_t pb = (size_t)plan.n_slots * kSlotStride * sizeof(float);
     if ((e = upload(&tasks, plan.tasks.data(), plan.tasks.size(), 0, s, &added)) != cudaSuccess ||
         (e = upload(&splits, plan.splits.data(), plan.splits.size(), 0, s, &added)) != cudaSuccess ||
+        (e = upload_split_state(plan, &slot_seg, &seg_done, s, &added)) != cudaSuccess ||
         (plan.n_slots > 0 && (e = cudaMalloc((void**)&partials, pb)) != cudaSuccess) ||
         (plan.n_slots > 0 && p.compensated && (e = cudaMalloc((void**)&pcomp, pb)) != cudaSuccess)) {
         cudaFree(tasks);
         cudaFree(splits);
+        cudaFree(slot_seg);
+        cudaFree(seg_done);
         cudaFree(partials);
         return cuda_fail(e, "replan: upload");
     }
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "replan: sync");
-    *bytes -= (int64_t)((d.n_tasks + 1) * sizeof(int4) + d.n_splits * sizeof(int4) +
+    *bytes -= (int64_t)((d.n_tasks + 1) * sizeof(int4) + d.n_splits * (sizeof(int4) + sizeof(unsigned int)) +
+                        d.n_slots * sizeof(int2) +
                         d.n_slots * kSlotStride * sizeof(float) * (d.partials_comp ? 2 : 1));
     *bytes += added + (int64_t)(pb * (pcomp ? 2 : 1));
     cudaFree(d.tasks);
     cudaFree(d.splits);
     cudaFree(d.partials);
     cudaFree(d.partials_comp);
+    cudaFree(d.slot_seg);
+    cudaFree(d.seg_done);
+    d.slot_seg = slot_seg;
+    d.seg_done = seg_done;
     d.partials_comp = pcomp;
     d.tasks = tasks;
     d.n_tasks = (int64_t)plan.tasks.size() - 1;

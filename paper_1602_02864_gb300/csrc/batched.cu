@@ -7,9 +7,8 @@
 // vector width, column chunks, compensation) form one group, and one
 // persistent launch of the task kernel runs the tasks of every entry of the
 // group, numbered one after the other: a warp finds its task's entry, then
-// takes that entry's matrix, X, Y, k and lane geometry.  The entries' split
-// rows are then combined by one more launch.  The entries' arguments travel
-// in the kernels' parameter space, so the call allocates nothing.
+// takes that entry's matrix, X, Y, k and lane geometry.  The entries' arguments
+// travel in the kernel's parameter space, so the call allocates nothing.
 #include <algorithm>
 #include <map>
 #include <memory>
@@ -53,7 +52,6 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
         int64_t tasks() const { return std::min(kMaxLaunchTasks, d->n_tasks - t0); }
     };
     std::map<std::tuple<int, int, int, int>, std::vector<Entry>> groups;
-    std::vector<Entry> all;
     for (int32_t i = 0; i < n; ++i) {
         const std::string who = "spmm_apply_batched: entry " + std::to_string(i);
         const spmm_mat* M = A[i];
@@ -88,7 +86,6 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
         en.ch = en.gm.ch;
         en.comp = d.partials_comp != nullptr || (M->params.compensated && d.n_slots == 0);
         groups[std::make_tuple(vmode, en.vec, en.ch, (int)en.comp)].push_back(en);
-        all.push_back(en);
     }
     // ---- one launch per group (and per kMaxBatch entries of it)
     auto M = std::make_unique<MultiArgs>();
@@ -129,6 +126,11 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
                 a.x_evict_last = H->params.x_evict_last;
                 a.compensated = en.comp ? 1 : 0;
                 a.partials_comp = d.partials_comp;
+                a.ctl = d.ctl;
+                a.splits = d.splits;
+                a.n_splits = d.n_splits;
+                a.slot_seg = d.slot_seg;
+                a.seg_done = d.seg_done;
                 M->off[q - c0] = tot;
                 tot += en.tasks();
                 wide = wide || (int64_t)k[en.i] * esize >= kWideRowBytes;
@@ -140,33 +142,11 @@ extern "C" int spmm_apply_batched(int32_t n, const spmm_mat_t* A, const void* co
             M->g.status = A[first.i]->status;
             M->g.wait_ns = kWaitNs;
             M->g.task_chunk = claim_chunk(tot, wide);
-            M->g.task_ctr = first.d->task_ctr;
-            cudaError_t e = cudaSuccess;
-            if (M->g.task_ctr) e = cudaMemsetAsync(M->g.task_ctr, 0, sizeof(unsigned long long), s);
-            if (e == cudaSuccess) e = launch_multi((int32_t)xtype, *M, first.vmode, first.vec, first.ch, first.comp, s);
+            M->g.ctl = first.d->ctl;
+            const cudaError_t e =
+                launch_multi((int32_t)xtype, *M, first.vmode, first.vec, first.ch, first.comp, s);
             if (e != cudaSuccess) return cuda_fail(e, "spmm_apply_batched: task kernel");
         }
-    }
-    // ---- the split rows of every entry
-    auto C = std::make_unique<CombineMulti>();
-    for (size_t c0 = 0; c0 < all.size(); c0 += kMaxBatch) {
-        const size_t c1 = std::min(all.size(), c0 + (size_t)kMaxBatch);
-        *C = CombineMulti{};
-        for (size_t q = c0; q < c1; ++q) {
-            const Entry& en = all[q];
-            if (en.d->n_splits == 0) continue;
-            CombineEntry& ce = C->ent[C->n++];
-            ce.splits = en.d->splits;
-            ce.n_splits = en.d->n_splits;
-            ce.partials = en.d->partials;
-            ce.pcomp = en.d->partials_comp;
-            ce.Y = static_cast<float*>(Y[en.i]);
-            ce.ldy = k[en.i];
-            ce.k = k[en.i];
-        }
-        if (C->n == 0) continue;
-        const cudaError_t e = launch_combine_multi(*C, s);
-        if (e != cudaSuccess) return cuda_fail(e, "spmm_apply_batched: combine kernel");
     }
     return SPMM_OK;
 }

@@ -8,11 +8,10 @@
 // and keeps a second copy of its column indices in which an entry of one of
 // the H most-referenced columns ("hot" columns) is ~slot, slot = the
 // column's rank (0 = most referenced).  A call whose X rows take 4 bytes
-// (k = 1 float32, k = 2 bf16/f16) first copies the H hot rows of X into a
-// packed buffer; the hot variant (one block of 24 warps per SM) copies that
-// buffer into shared memory once per block and gathers hot rows from there,
-// so only the other gathers use the L1-to-L2 request path, which bounds the
-// k = 1 product (78% busy on R-MAT).  The 8192 hottest columns take 21% of
+// (k = 1 float32, k = 2 bf16/f16) runs the hot variant (one block of 24 warps
+// per SM), whose blocks gather the H hot rows of X into shared memory at their
+// start and read them from there, so only the other gathers use the L1-to-L2
+// request path, which bounds the k = 1 product (78% busy on R-MAT).  The 8192 hottest columns take 21% of
 // R-MAT scale 24's entries; the product runs 10% faster with them (the
 // shared memory they take is L1 that the other gathers lose).  The sums and
 // their order are unchanged: only the address a row is read from differs.
@@ -83,43 +82,6 @@ int64_t hot_select(int64_t n_cols, const int32_t* col_idx, int64_t nnz, const in
         }
     });
     return H;
-}
-
-// Xh[s, 0:k] = X[hot_cols[s], 0:k], W-byte words (W divides the row bytes,
-// X's address and its row stride in bytes).
-template <typename W>
-__global__ void hot_gather_kernel(const char* __restrict__ X, int64_t ldx_bytes, const int32_t* __restrict__ hot_cols,
-                                  int64_t n_hot, int words_per_row, W* __restrict__ Xh) {
-    const int64_t total = n_hot * words_per_row;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t s = i / words_per_row;
-        const int w = (int)(i - s * words_per_row);
-        const int64_t c = hot_cols[s];
-        Xh[i] = __ldg(reinterpret_cast<const W*>(X + c * ldx_bytes) + w);
-    }
-}
-
-cudaError_t hot_gather(const DevCSR& d, const void* X, int64_t ldx, int32_t k, int esize, cudaStream_t s) {
-    if (d.n_hot <= 0) return cudaSuccess;
-    const int64_t row_bytes = (int64_t)k * esize, ld_bytes = ldx * esize;
-    const uintptr_t xa = (uintptr_t)X;
-    int w = 16;
-    while (w > esize && (row_bytes % w || ld_bytes % w || xa % w)) w >>= 1;
-    const int wpr = (int)(row_bytes / w);
-    const int64_t total = d.n_hot * wpr;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t want = (total + 255) / 256;
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sms * 8));
-    const char* Xc = static_cast<const char*>(X);
-    switch (w) {
-        case 16: hot_gather_kernel<uint4><<<grid, 256, 0, s>>>(Xc, ld_bytes, d.hot_cols, d.n_hot, wpr, (uint4*)d.xh); break;
-        case 8: hot_gather_kernel<uint2><<<grid, 256, 0, s>>>(Xc, ld_bytes, d.hot_cols, d.n_hot, wpr, (uint2*)d.xh); break;
-        case 4: hot_gather_kernel<uint32_t><<<grid, 256, 0, s>>>(Xc, ld_bytes, d.hot_cols, d.n_hot, wpr, (uint32_t*)d.xh); break;
-        default: hot_gather_kernel<uint16_t><<<grid, 256, 0, s>>>(Xc, ld_bytes, d.hot_cols, d.n_hot, wpr, (uint16_t*)d.xh); break;
-    }
-    return cudaGetLastError();
 }
 
 }  // namespace spmm

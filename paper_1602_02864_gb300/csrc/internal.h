@@ -47,6 +47,14 @@ constexpr int kColBufInts = kMaxTaskNnz + 8;          // 2080 bytes
 constexpr int kValBufBytes = (kMaxTaskNnz + 8) * 4;   // 2080 bytes
 constexpr int kRpBufLongs = kMaxTaskRows + 4;         // 544 bytes
 
+// Device words of one orientation: the next task to claim and the warps of the
+// running launch that have finished, both zero between launches (the last warp
+// resets them); and the next task of the launches that clear it beforehand
+// (rows_kernel.cuh, self_reset).
+struct TaskCtl {
+    unsigned int next, done, cleared_next, pad;
+};
+
 struct HostPlan {
     std::vector<int4> tasks;    // n_tasks + 1 (sentinel)
     std::vector<int4> splits;
@@ -82,17 +90,19 @@ struct DevCSR {
     float* partials_comp = nullptr; // compensation terms of the partials (compensated plans only)
     int64_t n_slots = 0;
     int32_t* perm = nullptr;        // SPMM_REORDER: original index of relabelled column c (n_cols)
-    unsigned long long* task_ctr = nullptr;   // task counter of dynamically scheduled launches
+    TaskCtl* ctl = nullptr;         // state that this orientation's launches pass on (zero between calls)
+    // the split and segments of each partial slot's row, and the segments that
+    // have arrived of each split row (FwdArgs::seg_done); not for streaming handles
+    int2* slot_seg = nullptr;
+    unsigned int* seg_done = nullptr;
     int32_t short_runs = 0;         // short-row runs over lane groups (spmm_opts.short_runs)
     // hot columns (hot.cu): col_hot is col_idx with ~slot for an entry in one
     // of the n_hot most-referenced columns, hot_cols[slot] that column; calls
-    // with X rows of at most 4 bytes copy the hot rows of X into xh (packed,
-    // kHotRowBytes each) and run the kernel variant that keeps them in
-    // shared memory
+    // with X rows of kHotRowBytes run the kernel variant that keeps the hot
+    // rows of X in shared memory
     int32_t* col_hot = nullptr;     // padded by 8 entries, like col_idx
     int32_t* hot_cols = nullptr;
     int64_t n_hot = 0;
-    void* xh = nullptr;
     double walk_eff[4] = {1.0, 1.0, 1.0, 1.0};   // HostPlan::walk_eff of the current plan
     std::vector<RowBlock> row_blocks;             // kRowBlocks runs of the current plan
 };
@@ -260,9 +270,6 @@ int apply_relabel_io(spmm_mat* A, int transpose, const void* X, int64_t ldx, int
 // first) and write col_idx with hot entries as ~slot to `encoded`; returns H
 int64_t hot_select(int64_t n_cols, const int32_t* col_idx, int64_t nnz, const int64_t* counts, int64_t max_hot,
                    std::vector<int32_t>& hot_cols, std::vector<int32_t>& encoded);
-// enqueue Xh[s, :] = X[hot_cols[s], :] (k elements of esize bytes) for the
-// n_hot hot columns of d
-cudaError_t hot_gather(const DevCSR& d, const void* X, int64_t ldx, int32_t k, int esize, cudaStream_t s);
 // hot rows that fit the shared memory of the hot kernel variant beside its
 // warps' staging buffers (value mode vmode, at most 4-byte rows); 0 if none
 int64_t hot_capacity(int vmode);
@@ -292,10 +299,16 @@ int apply_dev(const spmm_mat* A, int transpose, const void* X, int64_t ldx, int3
 // Y.  One run over all rows for streaming handles and plans without runs.
 int apply_dev_runs(const spmm_mat* A, int transpose, const void* X, int64_t ldx, int32_t k, int32_t xtype, float* Y,
                    int64_t ldy, cudaStream_t s, const std::function<int(int64_t, int64_t)>& rows_done);
-// the task counter for a launch over rows of k elements of xtype (reset on s;
-// nullptr for the static schedule) and the number of tasks per claim
-unsigned long long* task_counter(const DevCSR& d, int64_t n_tasks, int32_t k, int32_t xtype, cudaStream_t s,
-                                 cudaError_t* e, int32_t* chunk);
+// Split rows added by the warp that finishes them (FwdArgs::seg_done) or by a
+// second launch: inside while the task list is short.  Each segment's arrival
+// waits for its stores and an atomic; a second launch costs 2-3 us (R-MAT, k = 8
+// weighted: 406 tasks, 4 K vertices 12.5 -> 8.7 us; 5,002 tasks, 64 K 21.9 ->
+// 18.3; k = 1 15.8 -> 12.7; but k = 8, 512 K vertices, 36,046 tasks 67.7 ->
+// 70.8, 4 M vertices 400 -> 475).
+constexpr int64_t kCombineInsideTasks = 16384;
+inline bool combines_inside(const DevCSR& d) { return d.seg_done && d.n_tasks <= kCombineInsideTasks; }
+// tasks per claim of a launch over rows of k elements of xtype
+int32_t task_chunk_of(int64_t n_tasks, int32_t k, int32_t xtype);
 struct FwdArgs;
 // Lane geometry of one call: VEC elements per lane load (the widest vector
 // that divides k and keeps every X load and Y store aligned), CH column
@@ -342,20 +355,27 @@ struct FwdArgs {
     int32_t compensated;  // long rows / hub segments: compensated summation
     float* partials_comp; // compensation term of each segment partial (compensated only)
     // Dynamic scheduling: after its first task (static, one per warp), a warp
-    // claims the next task_chunk tasks, from W + task_chunk * atomicAdd(task_ctr,
-    // 1) on (W = warps in the grid); the counter is zero at launch.  nullptr:
-    // tasks t, t + W, t + 2W, ...
-    unsigned long long* task_ctr = nullptr;
-    int32_t task_chunk = 1;
+    // claims the next task_chunk tasks, from W + task_chunk * atomicAdd(&ctl->next,
+    // 1) on (W = warps in the grid).  task_chunk 0 or no ctl: tasks t, t + W, ...
+    TaskCtl* ctl = nullptr;
+    int32_t task_chunk = 0;
+    // split rows {row, segments, first slot} whose segments all lie in this
+    // call: the warp that finishes a row's last segment adds its partials.
+    // seg_done[i] counts row i's segments and is zero again once it is complete.
+    // nullptr: partials only, a second launch adds them.
+    const int4* splits = nullptr;
+    int64_t n_splits = 0;
+    const int2* slot_seg = nullptr;
+    unsigned int* seg_done = nullptr;
     // short-row runs over rows of several lanes: 1 = merge-based pieces per
     // lane group, 0 = each group walks whole rows
     int32_t merge_groups = 0;
     int32_t x_large = 0;   // X takes more than kLargeXBytes
-    // hot variant: a negative column index c names row ~c of the hot rows,
-    // hot_bytes (a multiple of 16) of them packed at Xh, copied into shared
-    // memory at the start of each block
-    const void* Xh = nullptr;
-    int64_t hot_bytes = 0;
+    // hot variant: a negative column index c names row ~c of the n_hot hot rows
+    // of X, row s of them being X's row hot_cols[s], which each block copies into
+    // shared memory at its start
+    const int32_t* hot_cols = nullptr;
+    int64_t n_hot = 0;
 };
 
 // X beyond the part of L2 that random gathers fill (64 MB of the GPU's L2: uniform
@@ -366,7 +386,7 @@ constexpr int64_t kLargeXBytes = 64ll << 20;
 // One launch over the tasks of several matrices (spmm_apply_batched): the
 // entries' arguments travel in the kernel's parameter space (no device
 // allocation); the tasks of entry e are numbers off[e] .. off[e+1]-1 of the
-// launch.  g holds the launch-wide fields: n_tasks (all entries), task_ctr,
+// launch.  g holds the launch-wide fields: n_tasks (all entries), ctl,
 // task_chunk, status, wait_ns.
 constexpr int kMaxBatch = 128;
 struct MultiArgs {
@@ -375,7 +395,7 @@ struct MultiArgs {
     int64_t off[kMaxBatch + 1];
     FwdArgs ent[kMaxBatch];
 };
-static_assert(sizeof(MultiArgs) <= 32000, "kernel parameter space holds at most 32764 bytes");
+static_assert(sizeof(MultiArgs) <= 32764, "kernel parameter space holds at most 32764 bytes");
 
 // Launches from a handle are scheduled dynamically.  Tasks over wide X rows
 // (at least kWideRowBytes bytes) vary a lot in time (gathers that miss L2)
@@ -418,7 +438,7 @@ cudaError_t launch_rows_f32_mg(const FwdArgs& a, int vmode, int vec, int ch, cud
 cudaError_t launch_rows_bf16_mg(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s);
 cudaError_t launch_rows_f16_mg(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s);
 // one lane per X row of at most 4 bytes with the hot rows in shared memory
-// (FwdArgs::Xh set)
+// (FwdArgs::hot_cols set)
 cudaError_t launch_rows_f32_hot(const FwdArgs& a, int vmode, int vec, cudaStream_t s);
 cudaError_t launch_rows_bf16_hot(const FwdArgs& a, int vmode, int vec, cudaStream_t s);
 cudaError_t launch_rows_f16_hot(const FwdArgs& a, int vmode, int vec, cudaStream_t s);
@@ -428,24 +448,6 @@ cudaError_t launch_rows_f16_hot(const FwdArgs& a, int vmode, int vec, cudaStream
 cudaError_t launch_rows_multi_f32(const MultiArgs& M, int vmode, int vec, int ch, bool comp, cudaStream_t s);
 cudaError_t launch_rows_multi_bf16(const MultiArgs& M, int vmode, int vec, int ch, bool comp, cudaStream_t s);
 cudaError_t launch_rows_multi_f16(const MultiArgs& M, int vmode, int vec, int ch, bool comp, cudaStream_t s);
-
-// combine.cu: the split rows of several matrices in one launch
-// (spmm_apply_batched); launch_combine_multi fills off[] and lanes_log2
-struct CombineEntry {
-    const int4* splits;
-    int64_t n_splits;
-    const float* partials;
-    const float* pcomp;     // compensation terms, or null
-    float* Y;
-    int64_t ldy;
-    int32_t k, lanes_log2;
-};
-struct CombineMulti {
-    int32_t n;
-    int64_t off[kMaxBatch + 1];
-    CombineEntry ent[kMaxBatch];
-};
-cudaError_t launch_combine_multi(CombineMulti& m, cudaStream_t s);
 
 // combine.cu: Y[row] = sum of the split row's partials in a fixed order.
 cudaError_t launch_combine(const int4* splits, int64_t n_splits, const float* partials, float* Y,

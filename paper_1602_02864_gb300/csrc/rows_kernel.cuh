@@ -7,7 +7,7 @@
 //
 // Persistent warps walk the task list (plan.cpp), claiming their next tasks
 // from an atomic counter (one task at a time for wide X rows, a few for narrow
-// ones; FwdArgs::task_ctr), or, without a counter, with a stride of the grid's
+// ones; FwdArgs::ctl), or, without a counter, with a stride of the grid's
 // warp count.  Each warp stages a task's column indices, values and row
 // pointers into shared memory with bulk asynchronous copies (cp.async.bulk,
 // completion on an mbarrier) one task ahead, so the copy of task i+1 overlaps
@@ -36,6 +36,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "combine.cuh"
 #include "internal.h"
 
 namespace spmm {
@@ -340,6 +341,22 @@ constexpr int min_blocks() {
     return (MG == 2 && VMODE == 0) ? 4 : two_blocks<VMODE, CH, ONE, MG>() ? 2 : SPMM_MIN_BLOCKS;
 }
 
+// A segment of a split row has its partial in a.partials: returns the row's
+// split if this was its last segment to arrive, -1 otherwise.  The arrival is a
+// release, not a full fence, which would empty L1 as well.
+__device__ __forceinline__ int segment_done(const FwdArgs& a, int slot, int lane) {
+    if (!a.seg_done || (int64_t)slot >= a.n_slots) return -1;
+    const int2 seg = a.slot_seg[slot];     // {split, segments of its row}
+    __syncwarp();                          // the lanes' parts of the partial, before the arrival
+    unsigned int before = 0;
+    if (lane == 0)                         // wraps to zero at the last arrival
+        asm volatile("atom.inc.release.gpu.global.u32 %0, [%1], %2;"
+                     : "=r"(before)
+                     : "l"(a.seg_done + seg.x), "r"((unsigned int)seg.y - 1u)
+                     : "memory");
+    return (int)__shfl_sync(0xffffffffu, before, 0) + 1 == seg.y ? seg.x : -1;
+}
+
 // ONE: one lane per X row (k == VEC, CH == 1); the lane geometry is then a
 // compile-time constant and short-row runs take the flat (k = 1) or, for X
 // rows of up to 8 bytes, the merge-based path.  MG != 0: several lanes per X
@@ -353,15 +370,28 @@ constexpr int warps_per_block() {
     return HOT ? kHotWarps : kWarpsPerBlock;
 }
 
-// HOT: one lane per X row of at most 4 bytes; a negative column index c
-// names row ~c of the hot rows of X, which the block copies into shared
-// memory (after its warps' staging buffers) before its first task, so those
-// gathers leave the L1-to-L2 request path alone (hot.cu).
+// HOT: one lane per X row of 4 bytes; a negative column index c names row ~c
+// of the hot rows of X, which the block gathers into shared memory (after its
+// warps' staging buffers) while its first tasks arrive, so those gathers leave
+// the L1-to-L2 request path alone (hot.cu).
+// Launches whose last warp resets the task counter: those of a few microseconds,
+// where a memset before each would cost 3 us (k = 1, 512 K vertices 40.9 ->
+// 37.4 us).  In the other instantiations the few instructions at the end
+// change the compiled task loop for the worse (FP16 k = 33, 700 K vertices 443 ->
+// 560 us), so their launches clear the counter first.
+template <bool ONE, bool HOT, bool SEG>
+constexpr bool self_reset() {
+    return ONE || HOT || SEG;
+}
+
+// SEG: the warp that finishes a split row's last segment adds the row's partials
+// (FwdArgs::seg_done); a variant of its own, since the other launches lose more
+// to the registers this takes than the second launch costs them.
 // MULTI: the tasks of several matrices (MultiArgs M, spmm_apply_batched),
 // numbered one after the other; every task takes the matrix, X, Y, k and
 // lane geometry of its own entry.  ga holds the launch-wide fields (task
 // count, counter, status, wait bound).
-template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG, bool HOT, bool MULTI>
+template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG, bool HOT, bool MULTI, bool SEG>
 __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) {
     static_assert(!MULTI || (!ONE && MG == 0 && !HOT), "batched launches use the generic row walk");
     static_assert(!ONE || CH == 1, "one lane per row needs CH == 1");
@@ -399,31 +429,10 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     uint64_t* bars = reinterpret_cast<uint64_t*>(wb + 2 * Lay::kBuf);
     const FwdArgs& a = ga;      // launch-wide fields (and, unless MULTI, the matrix's)
     const XT* hs = nullptr;     // hot rows of X in shared memory (HOT)
-    if constexpr (HOT) {
-        // one bulk copy of the packed hot rows, before any warp leaves
-        uint64_t* hbar = reinterpret_cast<uint64_t*>(smem + WPB * Lay::kWarp);
-        hs = reinterpret_cast<const XT*>(smem + WPB * Lay::kWarp + 16);
-        if (threadIdx.x == 0) {
-            mbar_init(hbar, 1);
-            fence_mbar_init();
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            mbar_arrive_expect_tx(hbar, (uint32_t)a.hot_bytes);
-            bulk_g2s(const_cast<XT*>(hs), a.Xh, (uint32_t)a.hot_bytes, hbar, policy_evict_last());
-        }
-        if (!mbar_wait_bounded(hbar, 0, a.wait_ns)) {
-            if (threadIdx.x == 0) atomicOr(a.status, kStatusTimeout);
-            // the copy may still be in flight: wait for it (bounded) before leaving
-            mbar_wait_bounded(hbar, 0, a.wait_ns);
-            return;
-        }
-    }
-
     const uint32_t n_tasks = (uint32_t)a.n_tasks;      // at most kMaxLaunchTasks
     const uint32_t W = gridDim.x * WPB;
     const uint32_t t = blockIdx.x * WPB + w;
-    if (t >= n_tasks) return;
+    if (!HOT && t >= n_tasks) return;
     if (lane == 0) {
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
@@ -495,9 +504,23 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
             issue_task<VMODE>(entry(e), x.a, desc_e0(x.end.x, x.end.y), wb + buf * Lay::kBuf, &bars[buf]);
     };
     Desc nx;
-    int ed = fetch(t, nx);
-    set_geometry(entry(ed));
-    stage(ed, nx, 0);
+    int ed = 0;
+    if (!HOT || t < n_tasks) {
+        ed = fetch(t, nx);
+        set_geometry(entry(ed));
+        stage(ed, nx, 0);
+    }
+    if constexpr (HOT) {
+        // the hot rows of X (one 4-byte word each) while the first tasks arrive
+        uint32_t* h4 = reinterpret_cast<uint32_t*>(smem + WPB * Lay::kWarp);
+        const uint32_t* x4 = reinterpret_cast<const uint32_t*>(a.X);
+        const uint64_t ld4 = (uint64_t)a.ldx / VEC;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < (int)a.n_hot; i += WPB * 32) h4[i] = __ldg(x4 + (uint64_t)a.hot_cols[i] * ld4);
+        hs = reinterpret_cast<const XT*>(h4);
+        __syncthreads();
+        if (t >= n_tasks) return;
+    }
     // the current task: first row, kind, low word of its first nonzero, nonzeros
     int2 d0;
     int e0, n;
@@ -511,10 +534,10 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     // counter by lane 0
     uint32_t cnext = 0, cend = 0;
     auto next_task = [&](uint32_t cur) -> uint32_t {
-        if (!a.task_ctr) return cur + W;
+        if (a.task_chunk == 0) return cur + W;
         if (cnext < cend) return cnext++;
         uint32_t v = 0;
-        if (lane == 0) v = atomicAdd(reinterpret_cast<unsigned int*>(a.task_ctr), 1u);
+        if (lane == 0) v = atomicAdd(self_reset<ONE, HOT, SEG>() ? &a.ctl->next : &a.ctl->cleared_next, 1u);
         cnext = W + __shfl_sync(0xffffffffu, v, 0) * (uint32_t)a.task_chunk;
         cend = cnext + a.task_chunk;
         return cnext++;
@@ -546,7 +569,8 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
         }
         phase ^= 1u << b;
 
-        // ---- compute task (d0, d1) from buffer b
+        int ready = -1;         // split row that this task completes
+        // ---- compute task (d0, e0, n) from buffer b
         if constexpr (MULTI) {
             if (cur != &entry(ed)) set_geometry(entry(ed));
         }
@@ -914,6 +938,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                         atomicOr(a.status, kStatusSlotRange);
                     }
                 }
+                if (SEG && d0.y < 0) ready = segment_done(a, -d0.y - 1, lane);
             } else {
                 // one long row or one hub segment: nonzeros g, g+G, ... per group
                 float acc[CH][VEC];
@@ -957,7 +982,13 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                     for (int c = 0; c < CH; ++c)
                         if (act[c]) store_y<VEC>(dst + (li + c * LANES) * VEC, acc[c]);
                 }
+                if (SEG && d0.y < 0) ready = segment_done(a, -d0.y - 1, lane);
             }
+        }
+        if (SEG && ready >= 0) {   // add its segments' partials, in segment order, into Y
+            __threadfence();    // the other warps' partials, after their arrivals
+            const FwdArgs& a = *cur;
+            combine_row(a.splits[ready], a.partials, a.Y, a.ldy, a.k, combine_lanes_log2(a.k), a.partials_comp, lane);
         }
         if (!more) break;
         take(nx);
@@ -969,21 +1000,45 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     }
 }
 
-template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG = 0, bool HOT = false>
+// The end of a warp: the launch's last one leaves the task counter at zero for
+// the next launch.  After a wait that ran out (in this launch or one not yet
+// reported) some segments may be missing, so it clears the arrivals too.
+__device__ __forceinline__ void warp_done(const FwdArgs& ga, const MultiArgs* M) {
+    if (!ga.ctl) return;
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    const unsigned int warps = gridDim.x * (blockDim.x >> 5);
+    unsigned int old = 0;
+    if (lane == 0) old = atomicInc(&ga.ctl->done, warps - 1);    // wraps to zero at the last
+    if (__shfl_sync(0xffffffffu, old, 0) != warps - 1) return;
+    if (lane == 0) ga.ctl->next = 0;
+    if (__ldcg(ga.status) == 0) return;
+    for (int e = 0; e < (M ? M->n : 1); ++e) {
+        const FwdArgs& a = M ? M->ent[e] : ga;
+        if (a.seg_done)
+            for (int64_t i = lane; i < a.n_splits; i += 32) a.seg_done[i] = 0;
+    }
+}
+
+template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG = 0, bool HOT = false, bool SEG = false>
 __global__ void __launch_bounds__(warps_per_block<HOT>() * 32, (HOT ? 1 : min_blocks<VMODE, CH, ONE, MG>()))
     rows_kernel(const __grid_constant__ FwdArgs a) {
-    rows_run<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT, false>(a, nullptr);
+    rows_run<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT, false, SEG>(a, nullptr);
+    if constexpr (self_reset<ONE, HOT, SEG>()) warp_done(a, nullptr);
 }
 
 // the tasks of up to kMaxBatch matrices in one launch (spmm_apply_batched);
 // two blocks per SM, so the per-task lane geometry fits in registers
 template <typename XT, int VMODE, int VEC, int CH, bool COMP>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, 2) rows_kernel_multi(const __grid_constant__ MultiArgs m) {
-    rows_run<XT, VMODE, VEC, CH, COMP, false, 0, false, true>(m.g, &m);
+    rows_run<XT, VMODE, VEC, CH, COMP, false, 0, false, true, true>(m.g, &m);
+    warp_done(m.g, &m);
 }
 
-template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG = 0, bool HOT = false>
+template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG = 0, bool HOT = false, bool SEG = false>
 cudaError_t launch_one(const FwdArgs& a, cudaStream_t s) {
+    if constexpr (!SEG && !COMP && !HOT)
+        if (a.seg_done) return launch_one<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT, true>(a, s);
     using Lay = Layout<VMODE>;
     constexpr int WPB = warps_per_block<HOT>();
     constexpr int kStage = WPB * Lay::kWarp;      // staging buffers of the block's warps
@@ -1001,10 +1056,10 @@ cudaError_t launch_one(const FwdArgs& a, cudaStream_t s) {
         // the hot variant asks for the whole opt-in shared memory (its hot rows fill what the staging leaves)
         const int want = HOT ? opt : kStage;
         if (e == cudaSuccess && want > 48 * 1024)
-            e = cudaFuncSetAttribute(rows_kernel<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT>,
+            e = cudaFuncSetAttribute(rows_kernel<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT, SEG>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, want);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, rows_kernel<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT>,
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, rows_kernel<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT, SEG>,
                                                               WPB * 32, want);
         setup = e;
         num_sms = sms;
@@ -1014,13 +1069,17 @@ cudaError_t launch_one(const FwdArgs& a, cudaStream_t s) {
     if (setup != cudaSuccess) return setup;
     size_t smem = kStage;
     if constexpr (HOT) {
-        smem += 16 + (size_t)a.hot_bytes;
-        if (smem > (size_t)max_smem || a.hot_bytes <= 0 || a.hot_bytes % 16) return cudaErrorInvalidValue;
+        smem += (size_t)a.n_hot * kHotRowBytes;
+        if (smem > (size_t)max_smem || a.n_hot <= 0) return cudaErrorInvalidValue;
+    }
+    if (!self_reset<ONE, HOT, SEG>() && a.task_chunk > 0) {
+        const cudaError_t e = cudaMemsetAsync(&a.ctl->cleared_next, 0, sizeof(unsigned int), s);
+        if (e != cudaSuccess) return e;
     }
     const int64_t want = (a.n_tasks + WPB - 1) / WPB;
     const int64_t cap = (int64_t)blocks_per_sm * num_sms;
     const dim3 grid((unsigned)(want < cap ? want : cap));
-    rows_kernel<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT><<<grid, WPB * 32, smem, s>>>(a);
+    rows_kernel<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT, SEG><<<grid, WPB * 32, smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -61,3 +61,50 @@ def test_every_task_claimed_once(sp, n_tasks, k):
         assert np.array_equal(Y.cpu().numpy().astype(np.float64), ref)
     finally:
         h.close()
+
+
+def _hubs(n_hubs, n_short, n_cols, seed):
+    """Rows of 513..3000 entries (split) among short ones."""
+    rng = np.random.default_rng(seed)
+    deg = rng.integers(0, 4, n_hubs + n_short)
+    deg[rng.choice(len(deg), n_hubs, replace=False)] = rng.integers(513, 3000, n_hubs)
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int64)
+    return rp, rng.integers(0, n_cols, rp[-1]).astype(np.int32)
+
+
+@pytest.mark.parametrize("n_hubs,n_short", [(1, 0), (40, 3000), (1000, 20000), (5000, 60000)])
+def test_split_rows_call_after_call(sp, n_hubs, n_short):
+    """Split rows are added by the launch itself on short task lists and by a second
+    launch on long ones; widths that take different kernels follow one another on one
+    handle, alone and in a batched call, and every sum is exact every time."""
+    import torch
+    n, m = n_hubs + n_short, 700
+    rp, ci = _hubs(n_hubs, n_short, m, n_hubs)
+    h = sp.SparseMatrix(n, m, rp, ci, None, transpose=True)
+    h2 = sp.SparseMatrix(n, m, rp, ci, None)
+    try:
+        assert h.info()["n_split_rows"] == n_hubs
+        assert (h.info()["n_tasks"] <= 16384) == (n_hubs <= 1000)
+        for k in (1, 64, 2, 3, 4, 8, 33, 16, 1, 8):
+            X = synth.dense(m, k, seed=k, mode="int")
+            Xg = torch.from_numpy(X).cuda()
+            ref = oracle.spmm(n, m, rp, ci, None, X)
+            for _ in range(2):
+                Y = torch.full((n, k), -1.0, device="cuda")
+                h.apply(Xg, Y=Y)
+                assert np.array_equal(Y.cpu().numpy().astype(np.float64), ref), k
+            Ys = [torch.full((n, k), -1.0, device="cuda") for _ in range(2)]
+            sp.spmm_apply_batched([h.handle, h2.handle], [Xg, Xg], Ys)
+            for Y in Ys:
+                assert np.array_equal(Y.cpu().numpy().astype(np.float64), ref), k
+            Xt = synth.dense(n, k, seed=k + 1, mode="int")
+            Yt = h.apply(torch.from_numpy(Xt).cuda(), transpose=True)
+            assert np.array_equal(Yt.cpu().numpy().astype(np.float64),
+                                  oracle.spmm(n, m, rp, ci, None, Xt, transpose=True)), k
+        sp.spmm_replan(h.handle, sp.spmm_opts(task_nnz=64, long_row=64))
+        X = synth.dense(m, 8, seed=9, mode="int")
+        Y = h.apply(torch.from_numpy(X).cuda())
+        assert np.array_equal(Y.cpu().numpy().astype(np.float64), oracle.spmm(n, m, rp, ci, None, X))
+    finally:
+        h.close()
+        h2.close()
