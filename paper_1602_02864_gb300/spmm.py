@@ -157,10 +157,32 @@ def _ptr(a) -> _P:
     return _P(a.data_ptr())   # torch tensor
 
 
-def _torch_dtype_code(t) -> int:
+# Filled on first use (importing this module does not import torch): dtype codes, and torch's
+# getters of the current device and of its current stream's handle.  torch.cuda.current_stream()
+# builds a Stream object (3 us, a fifth of a small product's call).
+_DTYPE_CODES: dict = {}
+_raw_stream = None
+_F32 = None
+
+
+def _load_torch():
+    global _raw_stream, _F32
     import torch
-    return {torch.float32: SPMM_F32, torch.bfloat16: SPMM_BF16, torch.float16: SPMM_F16,
-            torch.float64: SPMM_F64}[t.dtype]
+    _F32 = torch.float32
+    _DTYPE_CODES.update({torch.float32: SPMM_F32, torch.bfloat16: SPMM_BF16, torch.float16: SPMM_F16,
+                         torch.float64: SPMM_F64})
+    get = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if get is None:
+        _raw_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+    else:
+        device = torch.cuda.current_device
+        _raw_stream = lambda: get(device())  # noqa: E731
+
+
+def _torch_dtype_code(t) -> int:
+    if not _DTYPE_CODES:
+        _load_torch()
+    return _DTYPE_CODES[t.dtype]
 
 
 def _np_dtype_code(a) -> int:
@@ -173,8 +195,9 @@ def _np_dtype_code(a) -> int:
 
 def _stream_handle(stream) -> _P:
     if stream is None:
-        import torch
-        return _P(torch.cuda.current_stream().cuda_stream)
+        if _raw_stream is None:
+            _load_torch()
+        return _P(_raw_stream())
     if isinstance(stream, int):
         return _P(stream)
     return _P(stream.cuda_stream)
@@ -611,35 +634,37 @@ class SparseMatrix:
         vals = A.values if values is None else values
         return cls(A.n_rows, A.n_cols, A.row_ptr, A.col_idx, vals, transpose=transpose, **kw)
 
+    def _product(self, call, X, transpose, Y, stream):
+        shape, strides = X.shape, X.stride()
+        if len(shape) != 2 or strides[1] != 1:
+            raise ValueError("X must be 2-D with unit column stride")
+        xtype = _torch_dtype_code(X)
+        k = shape[1]
+        if Y is None:
+            Y = X.new_empty((self.n_cols if transpose else self.n_rows, k), dtype=_F32)
+            ldy = k
+        else:
+            if Y.dim() != 2 or Y.stride(1) != 1 or Y.dtype != _F32:
+                raise ValueError("Y must be a 2-D float32 tensor with unit column stride")
+            ldy = Y.stride(0)
+        if stream is None:
+            s = _raw_stream()
+        else:
+            s = stream if isinstance(stream, int) else stream.cuda_stream
+        rc = call(self.handle, X.data_ptr(), strides[0], k, xtype, Y.data_ptr(), ldy, SPMM_F32,
+                  1 if transpose else 0, s)
+        if rc:
+            _check(rc)
+        return Y
+
     def apply(self, X, transpose=False, Y=None, stream=None):
         """Y = A X (or A^T X).  X: 2-D CUDA tensor (float32/bfloat16/float16)
         with unit column stride; returns / fills a float32 CUDA tensor."""
-        import torch
-        if X.dim() != 2 or X.stride(1) != 1:
-            raise ValueError("X must be 2-D with unit column stride")
-        k = X.shape[1]
-        out_rows = self.n_cols if transpose else self.n_rows
-        if Y is None:
-            Y = torch.empty((out_rows, k), dtype=torch.float32, device=X.device)
-        if Y.dim() != 2 or Y.stride(1) != 1 or Y.dtype != torch.float32:
-            raise ValueError("Y must be a 2-D float32 tensor with unit column stride")
-        spmm_apply(self.handle, X, X.stride(0), k, _torch_dtype_code(X), Y, Y.stride(0), int(transpose), stream)
-        return Y
+        return self._product(_lib.spmm_apply, X, transpose, Y, stream)
 
     def apply_relabelled(self, X, transpose=False, Y=None, stream=None):
         """apply() with X and Y in the handle's vertex order (SPMM_RELABEL)."""
-        import torch
-        if X.dim() != 2 or X.stride(1) != 1:
-            raise ValueError("X must be 2-D with unit column stride")
-        k = X.shape[1]
-        out_rows = self.n_cols if transpose else self.n_rows
-        if Y is None:
-            Y = torch.empty((out_rows, k), dtype=torch.float32, device=X.device)
-        if Y.dim() != 2 or Y.stride(1) != 1 or Y.dtype != torch.float32:
-            raise ValueError("Y must be a 2-D float32 tensor with unit column stride")
-        spmm_apply_relabelled(self.handle, X, X.stride(0), k, _torch_dtype_code(X), Y, Y.stride(0), int(transpose),
-                              stream)
-        return Y
+        return self._product(_lib.spmm_apply_relabelled, X, transpose, Y, stream)
 
     def to_handle_order(self, M, out=None, stream=None):
         """M's rows (input vertex order) in the handle's order."""
