@@ -170,6 +170,7 @@ namespace spmm {
 struct PrCache {
     float *inv_deg = nullptr, *z = nullptr, *y = nullptr;
     double *part = nullptr, *scal = nullptr, *dres = nullptr;
+    unsigned int* done = nullptr;      // blocks of the running update that have finished (zero between)
     int32_t nblk = 0, dres_cap = 0;
     cudaStream_t s = nullptr;
     cudaGraphExec_t exec = nullptr;

@@ -8,8 +8,8 @@
 //
 // One iteration = the task kernel on A^T (k = 1, float32) + one fused
 // elementwise kernel (new ranks, the next z = x' * (1/L), FP64 per-block
-// partial sums of the L1 change and of the dangling mass) + a one-block kernel
-// adding the partials in a fixed order.  Iterations 2..iters are one CUDA
+// partial sums of the L1 change and of the dangling mass, added in a fixed order
+// by its last block).  Iterations 2..iters are one CUDA
 // graph; the handle keeps it with the workspace, so a later call with the
 // same x, damping and iteration count only launches it.  Ranks are float32;
 // every reduction is FP64 and run-to-run deterministic.
@@ -20,6 +20,7 @@
 namespace spmm {
 
 constexpr int kPrThreads = 256;
+constexpr int kPrUpdateFewer = 4;    // the update runs a quarter of the other passes' blocks: two an SM
 
 // Fixed-order block sum of a double (xor tree inside warps, then warp sums
 // added in warp order by thread 0).  Result valid in thread 0.
@@ -72,27 +73,46 @@ __global__ void pr_scale_kernel(const float* __restrict__ x, const float* __rest
     if (threadIdx.x == 0) part_dang[blockIdx.x] = s;
 }
 
+// A sum of floats as three floats, each holding what the one before rounded
+// away (Knuth's two-sum): 72 bits, so no less exact than an FP64 sum, on the
+// FP32 units (an FP64 addition and its conversion take 32 times as long here).
+struct FloatSum {
+    float s = 0.f, c = 0.f, d = 0.f;
+    static __device__ __forceinline__ float two_sum(float& a, float b) {
+        const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
+        a = t;
+        return e;
+    }
+    __device__ __forceinline__ void add(float v) { d = __fadd_rn(d, two_sum(c, two_sum(s, v))); }
+    __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)d); }
+};
+
 // x' = (1-d)/N + d*D/N + d*y, with D the dangling mass of x (scal[0]);
-// partials of sum |x' - x| and of the dangling mass of x'; z' = x' / L.
-// Float4 accesses; the per-element arithmetic is float32 and every group of
-// four is added to FP64 per-thread sums, then to FP64 block partials.
-__global__ void pr_update_kernel(const float* __restrict__ y, float* __restrict__ x, const float* __restrict__ inv,
-                                 int64_t n, double d, const double* __restrict__ scal, float* __restrict__ z,
-                                 double* __restrict__ part_res, double* __restrict__ part_dang) {
+// partials of sum |x' - x| and of the dangling mass of x'; z' = x' / L; the last
+// block to finish adds the partials in block order: scal[0] = the dangling mass
+// of x', *res_out = sum |x' - x|.  Float4 accesses, two in flight per thread; the
+// per-element arithmetic is float32, groups of four are added to per-thread sums
+// of 72 bits, those in FP64.  Bound by memory: with FP64 per-thread sums and 8
+// blocks an SM the FP64 units took two thirds of its 31.5 us on 4.2 M vertices,
+// and the final sum was a launch of its own (6.4 us); now 21.8 us with the sum (608 blocks 23.6,
+// 1216 35.2: each block adds its sums in FP64).
+__global__ void __launch_bounds__(kPrThreads)
+pr_update_kernel(const float* __restrict__ y, float* __restrict__ x, const float* __restrict__ inv, int64_t n, double d,
+                 double* __restrict__ scal, float* __restrict__ z, double* __restrict__ part_res,
+                 double* __restrict__ part_dang, double* __restrict__ res_out, unsigned int* __restrict__ done) {
     __shared__ double sh[32];
-    const float base = (float)((1.0 - d) / (double)n + d * scal[0] / (double)n);
+    __shared__ bool last;
+    const float base = (float)((1.0 - d) / (double)n + d * __ldcg(scal) / (double)n);
     const float df = (float)d;
-    double res = 0.0, dang = 0.0;
+    FloatSum res, dang;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool vec = ((((uintptr_t)x) | ((uintptr_t)y) | ((uintptr_t)z) | ((uintptr_t)inv)) & 15) == 0;
-    int64_t done = 0;
+    int64_t done_n = 0;
     if (vec) {
         const int64_t n4 = n >> 2;
-        for (int64_t i = tid; i < n4; i += stride) {
-            const float4 y4 = reinterpret_cast<const float4*>(y)[i];
-            float4 x4 = reinterpret_cast<const float4*>(x)[i];
-            const float4 v4 = reinterpret_cast<const float4*>(inv)[i];
+        auto four = [&](int64_t i, const float4 y4, float4 x4, const float4 v4) {
             float4 z4;
             float dg = 0.f, r = 0.f;
             r += pr_elem(y4.x, x4.x, v4.x, base, df, z4.x, dg);
@@ -101,42 +121,59 @@ __global__ void pr_update_kernel(const float* __restrict__ y, float* __restrict_
             r += pr_elem(y4.w, x4.w, v4.w, base, df, z4.w, dg);
             reinterpret_cast<float4*>(x)[i] = x4;
             reinterpret_cast<float4*>(z)[i] = z4;
-            res += (double)r;
-            dang += (double)dg;
+            res.add(r);
+            dang.add(dg);
+        };
+        const float4 *y_4 = reinterpret_cast<const float4*>(y), *v_4 = reinterpret_cast<const float4*>(inv);
+        const float4* x_4 = reinterpret_cast<const float4*>(x);
+        int64_t i = tid;
+        for (; i + stride < n4; i += 2 * stride) {
+            const float4 ya = y_4[i], xa = x_4[i], va = v_4[i];
+            const float4 yb = y_4[i + stride], xb = x_4[i + stride], vb = v_4[i + stride];
+            four(i, ya, xa, va);
+            four(i + stride, yb, xb, vb);
         }
-        done = n4 << 2;
+        if (i < n4) four(i, y_4[i], x_4[i], v_4[i]);
+        done_n = n4 << 2;
     }
-    for (int64_t i = done + tid; i < n; i += stride) {   // tail (or unaligned buffers)
+    for (int64_t i = done_n + tid; i < n; i += stride) {   // tail (or unaligned buffers)
         float xi = x[i], zi, dg = 0.f;
-        res += (double)pr_elem(y[i], xi, inv[i], base, df, zi, dg);
+        res.add(pr_elem(y[i], xi, inv[i], base, df, zi, dg));
         x[i] = xi;
         z[i] = zi;
-        dang += (double)dg;
+        dang.add(dg);
     }
-    const double s1 = block_sum(res, sh);
-    const double s2 = block_sum(dang, sh);
+    const double s1 = block_sum(res.value(), sh);
+    const double s2 = block_sum(dang.value(), sh);
     if (threadIdx.x == 0) {
         part_res[blockIdx.x] = s1;
         part_dang[blockIdx.x] = s2;
+        __threadfence();
+        last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;   // wraps to zero for the next launch
     }
-}
-
-// scal[0] = sum of the dangling partials; res_out (if given) = sum of the
-// residual partials; both in block order.
-__global__ void pr_reduce_kernel(const double* __restrict__ part_dang, const double* __restrict__ part_res,
-                                 int nparts, double* __restrict__ scal, double* __restrict__ res_out) {
-    __shared__ double sh[32];
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-        a += part_dang[i];
-        if (res_out) b += part_res[i];
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+        a += __ldcg(part_dang + i);
+        b += __ldcg(part_res + i);
     }
     const double sa = block_sum(a, sh);
     const double sb = block_sum(b, sh);
     if (threadIdx.x == 0) {
         scal[0] = sa;
-        if (res_out) *res_out = sb;
+        *res_out = sb;
     }
+}
+
+// scal[0] = sum of the dangling partials of pr_scale_kernel, in block order
+__global__ void pr_reduce_kernel(const double* __restrict__ part_dang, int nparts, double* __restrict__ scal) {
+    __shared__ double sh[32];
+    double a = 0.0;
+    for (int i = threadIdx.x; i < nparts; i += blockDim.x) a += part_dang[i];
+    const double sa = block_sum(a, sh);
+    if (threadIdx.x == 0) scal[0] = sa;
 }
 
 }  // namespace spmm
@@ -154,6 +191,7 @@ void pagerank_release(spmm_mat* A) {
     cudaFree(c.y);
     cudaFree(c.part);
     cudaFree(c.scal);
+    cudaFree(c.done);
     cudaFree(c.dres);
     cudaFree(c.xr);
     cudaFree(c.x0r);
@@ -178,7 +216,9 @@ static cudaError_t pr_reserve(PrCache& c, int64_t n, int32_t iters, int nblk) {
             (e = cudaMalloc((void**)&c.y, n * sizeof(float))) != cudaSuccess ||
             (e = cudaMalloc((void**)&c.part, 2 * (size_t)nblk * sizeof(double))) != cudaSuccess ||
             (e = cudaMalloc((void**)&c.scal, 8 * sizeof(double))) != cudaSuccess ||
-            (e = cudaStreamCreateWithFlags(&c.s, cudaStreamNonBlocking)) != cudaSuccess)
+            (e = cudaMalloc((void**)&c.done, sizeof(unsigned int))) != cudaSuccess ||
+            (e = cudaStreamCreateWithFlags(&c.s, cudaStreamNonBlocking)) != cudaSuccess ||
+            (e = cudaMemsetAsync(c.done, 0, sizeof(unsigned int), c.s)) != cudaSuccess)
             return e;
         c.nblk = nblk;
     }
@@ -259,15 +299,17 @@ extern "C" int spmm_pagerank(spmm_mat_t A, double damping, int32_t iters, float*
         // set-up outside the graph: 1/L, the start vector, z and its dangling mass
         pr_init_kernel<<<nblk, kPrThreads, 0, s>>>(A->fwd.row_ptr, n, c.inv_deg, x, x0);
         pr_scale_kernel<<<nblk, kPrThreads, 0, s>>>(x, c.inv_deg, n, c.z, c.part);
-        pr_reduce_kernel<<<1, kPrThreads, 0, s>>>(c.part, nullptr, nblk, c.scal, nullptr);
+        pr_reduce_kernel<<<1, kPrThreads, 0, s>>>(c.part, nblk, c.scal);
         if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "spmm_pagerank: init"); break; }
+        auto update = [&](int32_t t) {
+            pr_update_kernel<<<nblk / kPrUpdateFewer, kPrThreads, 0, s>>>(c.y, x, c.inv_deg, n, damping, c.scal, c.z,
+                                                                          c.part + nblk, c.part, c.dres + t, c.done);
+        };
         if (iters > 0) {
             // the first iteration runs outside the graph, so the task kernel's
             // one-time launch set-up (attributes, occupancy) happens before capture
             if ((rc = apply_dev(A, 1, c.z, 1, 1, SPMM_F32, c.y, 1, s)) != SPMM_OK) break;
-            pr_update_kernel<<<nblk, kPrThreads, 0, s>>>(c.y, x, c.inv_deg, n, damping, c.scal, c.z, c.part + nblk,
-                                                         c.part);
-            pr_reduce_kernel<<<1, kPrThreads, 0, s>>>(c.part, c.part + nblk, nblk, c.scal, c.dres);
+            update(0);
             if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "spmm_pagerank: first iteration"); break; }
         }
         if (iters > 1) {
@@ -287,9 +329,7 @@ extern "C" int spmm_pagerank(spmm_mat_t A, double damping, int32_t iters, float*
                 for (int32_t t = 1; t < iters && rc == SPMM_OK; ++t) {
                     rc = apply_dev(A, 1, c.z, 1, 1, SPMM_F32, c.y, 1, s);
                     if (rc != SPMM_OK) break;
-                    pr_update_kernel<<<nblk, kPrThreads, 0, s>>>(c.y, x, c.inv_deg, n, damping, c.scal, c.z,
-                                                                 c.part + nblk, c.part);
-                    pr_reduce_kernel<<<1, kPrThreads, 0, s>>>(c.part, c.part + nblk, nblk, c.scal, c.dres + t);
+                    update(t);
                 }
                 cudaGraph_t graph = nullptr;
                 cudaError_t ec = cudaStreamEndCapture(s, &graph);
