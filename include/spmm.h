@@ -88,7 +88,8 @@ typedef enum {
  *              (evict-last), 1 = evict-normal, 2 = evict-last; the
  *              streamed matrix is always read evict-first
  *   stream_slot_kib  streaming mode: staging slot size for column indices
- *              in KiB (two slots are used in turn)                 default 262144 (256 MiB)
+ *              in KiB (two slots are used in turn)                 default an eighth of the
+ *              indices, at least 16 MiB and at most 256 MiB
  *   debug_fail_block streaming mode, for tests: 1 + the block before
  *              which the streamer reports an injected copy failure and
  *              drains (0 = never)
@@ -230,8 +231,10 @@ typedef struct {
  * Section 3.6 argues memory is better spent on the dense side): the matrix is
  * NOT copied.  The handle borrows row_ptr, col_idx and values, pins them with
  * cudaHostRegister unless they are already pinned, and every spmm_apply
- * streams them to HBM in blocks of whole warp tasks through two staging slots
- * (the copy of one block overlaps the multiplication of the previous one).
+ * streams col_idx and values to HBM in blocks of whole warp tasks through two
+ * staging slots (the copy of one block overlaps the multiplication of the
+ * previous one).  A copy of row_ptr stays in HBM where 8 (n_rows + 3) bytes are
+ * free; otherwise it is streamed as well.
  * The caller must keep the arrays alive and unchanged until spmm_destroy.
  * Only Y = A X is available; X and Y stay in HBM.  Calls on one streaming
  * handle share its slots and must not overlap.

@@ -154,7 +154,7 @@ struct Params {
     int32_t long_row = 512;     // rows longer than this are split
     int32_t short_max = 63;     // rows with more nonzeros are "long"
     int32_t x_evict_last = 1;   // L2 policy of the X gathers (1 = evict-last)
-    int64_t slot_bytes = 256ll << 20;   // streaming staging slot (column indices)
+    int64_t slot_bytes = 0;     // streaming staging slot (column indices); 0 = by the matrix (stream.cu)
     int32_t fail_block = 0;
     int32_t compensated = 0;            // compensated sums for long rows and hub segments
     int32_t short_runs = 0;             // 0 automatic, 1 row walk, 2 pieces per lane group

@@ -9,8 +9,8 @@
 // X and Y stay in HBM, and the matrix flows over the host link in blocks of
 // whole warp tasks.  Two staging slots alternate: the copy of block b+1 runs
 // on a copy stream while the task kernel works on block b; events order each
-// slot's reuse.  The task list, split table and partials live in HBM as in
-// the resident mode, so results are identical to it.
+// slot's reuse.  The task list, row pointers, split table and partials live in
+// HBM as in the resident mode, so results are identical to it.
 //
 // The same pipeline serves a matrix kept in a file (spmm_create_file): each
 // block's column indices and values are first read from the file into one of
@@ -25,6 +25,8 @@
 #include "internal.h"
 
 namespace spmm {
+
+constexpr int64_t kSlotMinBytes = 16ll << 20, kSlotMaxBytes = 256ll << 20;
 
 // Cut the task list into blocks whose column-index range fits a slot.
 static void cut_blocks(const std::vector<int4>& tasks, int64_t n_rows, int64_t slot_nnz, std::vector<StreamBlock>& out,
@@ -89,7 +91,16 @@ int stream_setup(spmm_mat* A, const int64_t* row_ptr, const int32_t* col_idx, co
     HostPlan plan = build_plan(row_ptr, n, A->params);
     d.short_runs = A->params.short_runs;
     std::copy(plan.walk_eff, plan.walk_eff + 4, d.walk_eff);
-    const int64_t slot_nnz = std::max<int64_t>(A->params.slot_bytes / 4, 2 * kMaxTaskNnz + 16);
+    // unless the caller chose a slot: an eighth of the indices, in blocks of equal
+    // size, so that a block's product ends before its slot is wanted again and a
+    // call's last product is short; no less than a block's fixed cost is worth.
+    // R-MAT, 4 M vertices, 66 M entries, k = 4, us per call with slots of 8 / 16 / 32 /
+    // 64 / 128 MB: 1497 / 1431 / 1445 / 1478 / 1393, an eighth (33 MB) 1361; one of
+    // 256 MB and a short rest 1972 (with the row pointers streamed as well).
+    const int64_t slot_bytes = A->params.slot_bytes > 0
+                                   ? A->params.slot_bytes
+                                   : std::min(kSlotMaxBytes, std::max(kSlotMinBytes, nnz * 4 / 8 + 4096));
+    const int64_t slot_nnz = std::max<int64_t>(slot_bytes / 4, 2 * kMaxTaskNnz + 16);
     int64_t max_nnz = 0, max_rows = 0;
     cut_blocks(plan.tasks, n, slot_nnz, S.blocks, &max_nnz, &max_rows);
     S.slot_nnz = max_nnz + 16;
@@ -105,9 +116,21 @@ int stream_setup(spmm_mat* A, const int64_t* row_ptr, const int32_t* col_idx, co
         return cuda_fail(e, "streaming: pin row_ptr");
     if ((e = pin(col_idx, (size_t)nnz * 4, &S.reg_ci)) != cudaSuccess) return cuda_fail(e, "streaming: pin col_idx");
     if ((e = pin(values, (size_t)nnz * vsize, &S.reg_val)) != cudaSuccess) return cuda_fail(e, "streaming: pin values");
+    // the row pointers stay in HBM (padded as in the resident mode): a ninth of the
+    // bytes of a matrix of 16 entries a row, and one copy less per block (32 MB
+    // slots 1642 -> 1445 us).  Unless that memory is taken: then each block
+    // brings its own.
+    if (dmalloc((void**)&d.row_ptr, (size_t)(n + 3) * 8) == cudaSuccess) {
+        if ((e = cudaMemsetAsync(d.row_ptr + n + 1, 0, 16, s)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(d.row_ptr, row_ptr, (size_t)(n + 1) * 8, cudaMemcpyHostToDevice, s)) != cudaSuccess)
+            return cuda_fail(e, "streaming: row pointers");
+    } else {
+        cudaGetLastError();
+        d.row_ptr = nullptr;
+    }
     for (int i = 0; i < 2; ++i) {
         if ((e = dmalloc((void**)&S.slot_col[i], (size_t)S.slot_nnz * 4)) != cudaSuccess ||
-            (e = dmalloc((void**)&S.slot_rp[i], (size_t)S.slot_rows * 8)) != cudaSuccess ||
+            (!d.row_ptr && (e = dmalloc((void**)&S.slot_rp[i], (size_t)S.slot_rows * 8)) != cudaSuccess) ||
             (vsize > 0 && (e = dmalloc(&S.slot_val[i], (size_t)S.slot_nnz * vsize)) != cudaSuccess))
             return cuda_fail(e, "streaming: staging slots");
     }
@@ -149,7 +172,7 @@ int stream_setup(spmm_mat* A, const int64_t* row_ptr, const int32_t* col_idx, co
             *bytes += (int64_t)d.n_slots * kSlotStride * sizeof(float);
         }
     }
-    S.bytes_per_apply = nnz * 4 + (int64_t)(nnz * vsize) + (n + 1) * 8;
+    S.bytes_per_apply = nnz * 4 + (int64_t)(nnz * vsize) + (d.row_ptr ? 0 : (n + 1) * 8);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "streaming: set-up");
     return SPMM_OK;
 }
@@ -236,7 +259,8 @@ int stream_apply(const spmm_mat* A, const void* X, int64_t ldx, int32_t k, int32
         if (vmode && (e = cudaMemcpyAsync(S.slot_val[slot], src_val, (size_t)(b.c1 - b.c0) * vsize,
                                           cudaMemcpyHostToDevice, S.copy)) != cudaSuccess)
             break;
-        if ((e = cudaMemcpyAsync(S.slot_rp[slot], S.h_row_ptr + b.r0, (size_t)(b.r1 - b.r0) * 8,
+        if (!d.row_ptr &&
+            (e = cudaMemcpyAsync(S.slot_rp[slot], S.h_row_ptr + b.r0, (size_t)(b.r1 - b.r0) * 8,
                                  cudaMemcpyHostToDevice, S.copy)) != cudaSuccess)
             break;
         if ((e = cudaEventRecord(S.copied[slot], S.copy)) != cudaSuccess) break;
@@ -245,7 +269,7 @@ int stream_apply(const spmm_mat* A, const void* X, int64_t ldx, int32_t k, int32
         // rebased views: global index i of the block lives at slot offset i - c0 (or i - r0)
         a.col_idx = S.slot_col[slot] - b.c0;
         a.val = vmode ? static_cast<const void*>(static_cast<const char*>(S.slot_val[slot]) - b.c0 * vsize) : nullptr;
-        a.row_ptr = S.slot_rp[slot] - b.r0;
+        a.row_ptr = d.row_ptr ? d.row_ptr : S.slot_rp[slot] - b.r0;
         a.tasks = d.tasks + b.t0;
         a.n_tasks = b.t1 - b.t0;
         a.ctl = d.ctl;

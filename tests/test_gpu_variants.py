@@ -108,3 +108,23 @@ def test_split_rows_call_after_call(sp, n_hubs, n_short):
     finally:
         h.close()
         h2.close()
+
+
+def test_streaming_default_slots(sp):
+    """Enough entries for several blocks of the default slot size (16 MiB and more): the
+    resident result bit for bit, call after call, at the widths that take other kernels."""
+    import torch
+    A = synth.rmat_csr(20, n_edges=14 << 20, seed=8)
+    assert A.nnz * 4 > 2 * (16 << 20)
+    hs = sp.SparseMatrix(A.n_rows, A.n_cols, A.row_ptr, A.col_idx, None, streaming=True)
+    hr = sp.SparseMatrix(A.n_rows, A.n_cols, A.row_ptr, A.col_idx, None)
+    try:
+        for k in (1, 4, 33):
+            X = torch.from_numpy(synth.dense(A.n_cols, k, seed=k)).cuda()
+            Yr = hr.apply(X)
+            for _ in range(3):
+                assert torch.equal(hs.apply(X), Yr), k
+        hs.sync_status()
+    finally:
+        hs.close()
+        hr.close()
