@@ -438,6 +438,10 @@ cudaError_t launch_rows_f16_one(const FwdArgs& a, int vmode, int vec, int ch, cu
 cudaError_t launch_rows_f32_mg(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s);
 cudaError_t launch_rows_bf16_mg(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s);
 cudaError_t launch_rows_f16_mg(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s);
+// a whole warp per X row of two chunks (ch == 2: vec == 1, k > 32)
+cudaError_t launch_rows_f32_warp(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s);
+cudaError_t launch_rows_bf16_warp(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s);
+cudaError_t launch_rows_f16_warp(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s);
 // one lane per X row of at most 4 bytes with the hot rows in shared memory
 // (FwdArgs::hot_cols set)
 cudaError_t launch_rows_f32_hot(const FwdArgs& a, int vmode, int vec, cudaStream_t s);

@@ -7,6 +7,7 @@ namespace spmm {
 cudaError_t launch_rows_f16(const FwdArgs& a, int vmode, int vec, int ch, cudaStream_t s) {
     if (a.hot_cols && ch == 1 && a.lanes_log2 == 0) return launch_rows_f16_hot(a, vmode, vec, s);
     if (ch == 1 && a.lanes_log2 == 0) return launch_rows_f16_one(a, vmode, vec, ch, s);
+    if (ch == 2) return launch_rows_f16_warp(a, vmode, vec, ch, s);
     if (a.merge_groups) return launch_rows_f16_mg(a, vmode, vec, ch, s);
     return launch_rows_t<__half, false>(a, vmode, vec, ch, s);
 }

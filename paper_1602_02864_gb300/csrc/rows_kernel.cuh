@@ -325,8 +325,8 @@ __device__ __forceinline__ void issue_task(const FwdArgs& a, const int4 d0, int6
 // shared memory and leave L1 next to nothing (weighted R-MAT, 4 M vertices,
 // FP32, ms with three -> two: k = 1 0.395 -> 0.252, k = 2 0.424 -> 0.291, k = 8
 // 0.684 -> 0.440; BF16 X, k = 16 0.771 -> 0.622; 2 M, k = 64 1.081 -> 0.834), and
-// for rows on two chunks of single elements (FP16, k = 33, 700 K vertices
-// 0.492 -> 0.443).  Pattern rows on one chunk lose (k = 8, 8 M vertices 0.90 ->
+// for rows on two chunks of single elements, whose walk keeps 16 rows' loads
+// in flight (MG == 4; with three blocks it spills).  Pattern rows on one chunk lose (k = 8, 8 M vertices 0.90 ->
 // 1.03 ms, k = 32, 4 M 1.03 -> 1.19).  The weighted group merge comes in both
 // forms (MG == 1, MG == 3): lanes of 16 bytes run faster with three blocks while X
 // fits L2 (k = 16, 37 MB of X: 0.152 against 0.162 ms) and with two beyond
@@ -334,7 +334,7 @@ __device__ __forceinline__ void issue_task(const FwdArgs& a, const int4 d0, int6
 // 0.510 against 0.433).
 template <int VMODE, int CH, bool ONE, int MG>
 constexpr bool two_blocks() {
-    return (VMODE != 0 && MG == 0) || MG == 3 || CH == 2;
+    return (VMODE != 0 && MG == 0) || MG == 3 || MG == 4;
 }
 template <int VMODE, int CH, bool ONE, int MG>
 constexpr int min_blocks() {
@@ -362,7 +362,13 @@ __device__ __forceinline__ int segment_done(const FwdArgs& a, int slot, int lane
 // rows of up to 8 bytes, the merge-based path.  MG != 0: several lanes per X
 // row (CH == 1) and short-row runs merge-based over lane groups, with 3
 // blocks per SM and 4 nonzeros in flight per group (MG == 1), 4 blocks and 2 in
-// flight (MG == 2) or 2 blocks and 8 in flight (MG == 3).
+// flight (MG == 2) or 2 blocks and 8 in flight (MG == 3).  MG == 4: a whole warp
+// per X row of two chunks (odd k above 32), which takes a task's nonzeros as one
+// stream, 8 + 8 rows in flight across the ends of the task's rows: the row walk
+// has one row's loads in flight, and half of R-MAT's rows have fewer than four
+// (FP16 k = 33, 700 K vertices 0.445 -> 0.378 ms, FP32 k = 33, 1 M 0.731 ->
+// 0.551).  Rows on one chunk gain nothing (FP32 k = 31, 512 K 0.201 -> 0.210),
+// nor does k = 64 on 32 lanes of two elements (2 M 0.795 -> 0.850).
 // Warps per block: kWarpsPerBlock, or kHotWarps in one block per SM for the
 // instantiations that keep the hot rows of X in shared memory (HOT).
 template <bool HOT>
@@ -395,7 +401,7 @@ template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG, 
 __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) {
     static_assert(!MULTI || (!ONE && MG == 0 && !HOT), "batched launches use the generic row walk");
     static_assert(!ONE || CH == 1, "one lane per row needs CH == 1");
-    static_assert(MG == 0 || (!ONE && CH == 1), "merge over lane groups needs several lanes and CH == 1");
+    static_assert(MG == 0 || (!ONE && CH == (MG == 4 ? 2 : 1)), "merge over lane groups: several lanes, one chunk");
     static_assert(!HOT || (ONE && MG == 0 && VEC * sizeof(XT) <= 4), "hot rows in shared memory: <= 4-byte rows");
     constexpr int WPB = warps_per_block<HOT>();
     constexpr bool kFlat = ONE && VEC == 1 && SPMM_K1_FLAT;
@@ -403,7 +409,9 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     // (mostly gathered from DRAM) the row-per-lane walk measured faster
     constexpr bool kMerge = ONE && !kFlat && SPMM_MERGE && VEC * sizeof(XT) <= 8;
     // the same over lane groups, for rows that need several lanes (MG)
-    constexpr bool kMergeG = MG != 0;
+    constexpr bool kMergeG = MG != 0 && MG != 4;
+    // a whole warp per X row: the run's nonzeros one after the other
+    constexpr bool kWholeWarp = MG == 4;
     using Lay = Layout<VMODE>;
     // nonzeros in flight per lane group
     constexpr int kBytes = VEC * CH * (int)sizeof(XT);
@@ -421,8 +429,11 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     // shared memory when they are used and the task state fits few registers, so
     // 4 in flight spill neither with values (2 before: k = 16 weighted, 37 MB of
     // X 0.168 -> 0.152 ms) nor without; 6 do (0.211).
-    constexpr int kUW = MG == 3 ? 2 * SPMM_MERGE_WIDE_UNROLL : MG == 1 ? SPMM_MERGE_WIDE_UNROLL : 2;
-    constexpr int UW = U < kUW ? U : kUW;
+    constexpr int kUW = MG == 4   ? 8
+                        : MG == 3 ? 2 * SPMM_MERGE_WIDE_UNROLL
+                        : MG == 1 ? SPMM_MERGE_WIDE_UNROLL
+                                  : 2;
+    constexpr int UW = MG == 4 ? kUW : U < kUW ? U : kUW;
     extern __shared__ __align__(128) unsigned char smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char* wb = smem + w * Lay::kWarp;
@@ -477,7 +488,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     uint64_t xpol = 0;
     const FwdArgs* cur = &a;    // the entry of the task being computed
     auto set_geometry = [&](const FwdArgs& E) {
-        lg = ONE ? 0 : E.lanes_log2;
+        lg = ONE ? 0 : kWholeWarp ? 5 : E.lanes_log2;
         LANES = 1 << lg;
         G = 32 >> lg;
         g = lane >> lg;
@@ -827,7 +838,87 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
 #pragma unroll
                 for (int v = 0; v < VEC; ++v) head[v] += __shfl_up_sync(0xffffffffu, tail[v], LANES);
                 if (hrow >= 0 && act[0]) store_y<VEC>(a.Y + (int64_t)(d0.x + hrow) * a.ldy + li * VEC, head);
-            } else if (!kFlat && !kMerge && !kMergeG && d0.y > 0) {
+            } else if (kWholeWarp && d0.y > 0) {
+                // run of short rows, 32 lanes per X row: the warp takes the task's
+                // nonzeros in order, UW rows of X requested while the UW before are
+                // added, across the ends of rows; no bounds are checked inside a
+                // whole batch, and every branch is the warp's.  Each row's sum is
+                // that of the row walk.
+                const int nr = d0.y;
+                int r = 0, re = st.rp(1);
+                float acc[CH][VEC];
+#pragma unroll
+                for (int c = 0; c < CH; ++c)
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) acc[c][v] = 0.f;
+                auto end_row = [&]() {
+                    float* dst = a.Y + (int64_t)(d0.x + r) * a.ldy;
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) {
+                        if (act[c]) store_y<VEC>(dst + (li + c * 32) * VEC, acc[c]);
+#pragma unroll
+                        for (int v = 0; v < VEC; ++v) acc[c][v] = 0.f;
+                    }
+                    ++r;
+                };
+                auto add1 = [&](XVec<XT, VEC>(&x)[CH], int i) {
+                    const float av = staged_val<VMODE>(st.val, i);
+#pragma unroll
+                    for (int c = 0; c < CH; ++c)
+#pragma unroll
+                        for (int v = 0; v < VEC; ++v) acc[c][v] = fmaf(av, x[c].get(v), acc[c][v]);
+                };
+                auto load1 = [&](XVec<XT, VEC>(&x)[CH], int i) {
+                    const int64_t cidx = st.col[i];
+#pragma unroll
+                    for (int c = 0; c < CH; ++c)
+                        if (act[c]) gather(x[c], cidx, c * 32 * VEC);
+                };
+                auto load = [&](XVec<XT, VEC>(&x)[UW][CH], int i) {
+#pragma unroll
+                    for (int u = 0; u < UW; ++u) load1(x[u], i + u);
+                };
+                auto add = [&](XVec<XT, VEC>(&x)[UW][CH], int i) {
+                    if (i + UW <= re) {            // all in the current row
+#pragma unroll
+                        for (int u = 0; u < UW; ++u) add1(x[u], i + u);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < UW; ++u) {
+                            while (i + u >= re) {
+                                end_row();
+                                re = st.rp(r + 1);
+                            }
+                            add1(x[u], i + u);
+                        }
+                    }
+                };
+                XVec<XT, VEC> xa[UW][CH], xb[UW][CH];
+                const int full = n - n % UW;
+                if (full > 0) load(xa, 0);
+                int i = 0;
+                for (; i < full; i += 2 * UW) {
+                    if (i + UW < full) load(xb, i + UW);
+                    add(xa, i);
+                    if (i + UW < full) {
+                        if (i + 2 * UW < full) load(xa, i + 2 * UW);
+                        add(xb, i + UW);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < UW - 1; ++u)
+                    if (full + u < n) load1(xa[u], full + u);
+#pragma unroll
+                for (int u = 0; u < UW - 1; ++u)
+                    if (full + u < n) {
+                        while (full + u >= re) {
+                            end_row();
+                            re = st.rp(r + 1);
+                        }
+                        add1(xa[u], full + u);
+                    }
+                while (r < nr) end_row();
+            } else if (!kFlat && !kMerge && !kMergeG && !kWholeWarp && d0.y > 0) {
                 // run of short rows: lane group g owns rows g, g+G, ...
                 const int nr = d0.y;
                 for (int j = g; j < nr; j += G) {
@@ -1164,6 +1255,13 @@ cudaError_t launch_rows_t(const FwdArgs& a, int vmode, int vec, int ch, cudaStre
                              : launch_one<XT, VM, V, C, false, ONE, MG>(a, s);
     if constexpr (MG == 2) {     // float pattern rows of 4-element lanes only
         if constexpr (sizeof(XT) == 4) { SPMM_LAUNCH(0, 4, 1) }
+    } else if constexpr (MG == 4) {   // a whole warp per X row, two chunks of single elements
+        if constexpr (sizeof(XT) == 4) {
+            SPMM_LAUNCH(0, 1, 2) SPMM_LAUNCH(1, 1, 2)
+        } else {
+            constexpr int VM3 = std::is_same<XT, __half>::value ? 3 : 2;
+            SPMM_LAUNCH(0, 1, 2) SPMM_LAUNCH(1, 1, 2) SPMM_LAUNCH(VM3, 1, 2)
+        }
     } else if constexpr (MG == 3) {   // staged values only
         if constexpr (sizeof(XT) == 4) {
             SPMM_LAUNCH(1, 4, 1) SPMM_LAUNCH(1, 2, 1) SPMM_LAUNCH(1, 1, 1)
@@ -1194,14 +1292,13 @@ cudaError_t launch_rows_t(const FwdArgs& a, int vmode, int vec, int ch, cudaStre
         }
     } else {
         if constexpr (sizeof(XT) == 4) {
-            SPMM_LAUNCH(0, 4, 1) SPMM_LAUNCH(0, 2, 1) SPMM_LAUNCH(0, 1, 1) SPMM_LAUNCH(0, 1, 2)
-            SPMM_LAUNCH(1, 4, 1) SPMM_LAUNCH(1, 2, 1) SPMM_LAUNCH(1, 1, 1) SPMM_LAUNCH(1, 1, 2)
+            SPMM_LAUNCH(0, 4, 1) SPMM_LAUNCH(0, 2, 1) SPMM_LAUNCH(0, 1, 1)
+            SPMM_LAUNCH(1, 4, 1) SPMM_LAUNCH(1, 2, 1) SPMM_LAUNCH(1, 1, 1)
         } else {
             constexpr int VM3 = std::is_same<XT, __half>::value ? 3 : 2;
-            SPMM_LAUNCH(0, 8, 1) SPMM_LAUNCH(0, 4, 1) SPMM_LAUNCH(0, 2, 1) SPMM_LAUNCH(0, 1, 1) SPMM_LAUNCH(0, 1, 2)
-            SPMM_LAUNCH(1, 8, 1) SPMM_LAUNCH(1, 4, 1) SPMM_LAUNCH(1, 2, 1) SPMM_LAUNCH(1, 1, 1) SPMM_LAUNCH(1, 1, 2)
+            SPMM_LAUNCH(0, 8, 1) SPMM_LAUNCH(0, 4, 1) SPMM_LAUNCH(0, 2, 1) SPMM_LAUNCH(0, 1, 1)
+            SPMM_LAUNCH(1, 8, 1) SPMM_LAUNCH(1, 4, 1) SPMM_LAUNCH(1, 2, 1) SPMM_LAUNCH(1, 1, 1)
             SPMM_LAUNCH(VM3, 8, 1) SPMM_LAUNCH(VM3, 4, 1) SPMM_LAUNCH(VM3, 2, 1) SPMM_LAUNCH(VM3, 1, 1)
-            SPMM_LAUNCH(VM3, 1, 2)
         }
     }
 #undef SPMM_LAUNCH

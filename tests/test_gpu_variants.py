@@ -128,3 +128,37 @@ def test_streaming_default_slots(sp):
     finally:
         hs.close()
         hr.close()
+
+
+@pytest.mark.parametrize("xdtype", ["float32", "bfloat16", "float16"])
+@pytest.mark.parametrize("k", [33, 47, 63])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_whole_warp_rows(sp, xdtype, k, weighted):
+    """Odd widths above 32 (a warp per X row): runs with empty rows at both ends, tasks of 0 to
+    512 entries around the batches of 8, against the oracle; small integers exactly."""
+    import torch
+    rng = np.random.default_rng(k)
+    deg = np.concatenate([[0, 0, 7, 8, 9, 0, 15, 16, 17, 1], rng.integers(0, 3, 500), np.zeros(70, np.int64),
+                          rng.integers(0, 64, 600), [63] * 64, [0, 600, 0, 64], rng.integers(0, 2, 131), [0]])
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int64)
+    n, m = len(deg), 3001
+    ci = rng.integers(0, m, rp[-1]).astype(np.int32)
+    vals = rng.random(rp[-1]).astype(np.float32) if weighted else None
+    h = sp.SparseMatrix(n, m, rp, ci, vals, transpose=True)
+    try:
+        for tr in (False, True):
+            rows, cols = (m, n) if tr else (n, m)
+            Xi = synth.dense(cols, k, seed=1, mode="int")
+            Xf = torch.from_numpy(synth.dense(cols, k, seed=2)).to(getattr(torch, xdtype))
+            Xf_h = Xf.float().numpy()
+            Y = torch.full((rows, k), np.nan, device="cuda")
+            h.apply(Xf.cuda(), transpose=tr, Y=Y)
+            ref = oracle.spmm(n, m, rp, ci, vals, Xf_h, transpose=tr)
+            scale = oracle.spmm(n, m, rp, ci, vals, np.abs(Xf_h), transpose=tr)
+            assert np.all(np.abs(Y.cpu().numpy() - ref) <= 1e-5 * scale + 1e-30)
+            if not weighted:
+                Yi = h.apply(torch.from_numpy(Xi).to(getattr(torch, xdtype)).cuda(), transpose=tr)
+                assert np.array_equal(Yi.cpu().numpy().astype(np.float64),
+                                      oracle.spmm(n, m, rp, ci, None, Xi, transpose=tr))
+    finally:
+        h.close()
