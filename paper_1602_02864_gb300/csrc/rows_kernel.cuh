@@ -876,7 +876,8 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                 // nonzeros in order, UW rows of X requested while the UW before are
                 // added, across the ends of rows; no bounds are checked inside a
                 // whole batch, and every branch is the warp's.  Each row's sum is
-                // that of the row walk.
+                // that of the row walk, and no row beyond the run is written, whatever
+                // a caller's task list says (spmm_apply_csr_static).
                 const int nr = d0.y;
                 int r = 0, re = st.rp(1);
                 float acc[CH][VEC];
@@ -918,7 +919,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
                     } else {
 #pragma unroll
                         for (int u = 0; u < UW; ++u) {
-                            while (i + u >= re) {
+                            while (i + u >= re && r < nr) {
                                 end_row();
                                 re = st.rp(r + 1);
                             }
@@ -944,7 +945,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
 #pragma unroll
                 for (int u = 0; u < UW - 1; ++u)
                     if (full + u < n) {
-                        while (full + u >= re) {
+                        while (full + u >= re && r < nr) {
                             end_row();
                             re = st.rp(r + 1);
                         }
