@@ -454,16 +454,15 @@ def workload_streaming(args):
     for _ in range(args.warmup):
         h.apply(X, Y=Y)
     # the host link can be shared with other jobs: time the streamed calls
-    # interleaved with a copy-only pass over the same host arrays
+    # interleaved with a copy-only pass over the same host array (the column
+    # indices; the row pointers stay on the device with the handle)
     ci = torch.from_numpy(A.col_idx).view(torch.uint8)
-    rp = torch.from_numpy(A.row_ptr).view(torch.uint8)
     stage = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
 
     def copy_only():
-        for src in (ci, rp):
-            for off in range(0, src.numel(), 256 << 20):
-                n = min(256 << 20, src.numel() - off)
-                stage[:n].copy_(src[off:off + n], non_blocking=True)
+        for off in range(0, ci.numel(), 256 << 20):
+            n = min(256 << 20, ci.numel() - off)
+            stage[:n].copy_(ci[off:off + n], non_blocking=True)
     ms_list, copy_list = [], []
     for _ in range(args.steps):
         ms_list.append(event_ms(lambda: h.apply(X, Y=Y), 1))
@@ -474,7 +473,7 @@ def workload_streaming(args):
     peak_after = max((1 << 30) / (event_ms(lambda: dbuf2.copy_(buf2, non_blocking=True), 1) / 1e3) / 1e9
                      for buf2, dbuf2 in [(torch.empty(1 << 30, dtype=torch.uint8).pin_memory(),
                                           torch.empty(1 << 30, dtype=torch.uint8, device="cuda"))] for _ in range(5))
-    link_bytes = nnz * 4 + (N + 1) * 8
+    link_bytes = nnz * 4
     # resident mode on the same matrix for context
     hr = spmm.SparseMatrix(N, N, A.row_ptr, A.col_idx, None)
     Yr = torch.empty_like(Y)
@@ -500,7 +499,7 @@ def workload_streaming(args):
                                "frac_of_copy_only": copy_ms / ms,
                                "bytes_per_call": link_bytes,
                                "note": "steps alternate a streamed call and a copy-only pass over the same "
-                                       "pinned host arrays (the host link may be shared)"},
+                                       "pinned host array of column indices (the host link may be shared)"},
                       "resident_ms": ms_res, "bit_identical_to_resident": same,
                       "sampled_rows_max_err_over_absprod": err, "sampled_rows": int(len(rows)),
                       "n": N, "nnz": nnz, "setup_s": {"generate": round(t_gen, 1), "create": round(t_create, 1)}})
@@ -1063,15 +1062,14 @@ def main():
     Y = {k: torch.empty((N, k), dtype=torch.float32, device=dev) for k in ks}
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device=dev)
     stream = torch.cuda.current_stream()
-    # per product: the task kernel, the combine pass (if rows are split) and,
-    # for 4-byte X rows (k = 1 float32), the packing of the hot X rows
-    launches_per_apply = 1 + (1 if info["n_split_rows"] > 0 else 0)
-    sweep_launches = sum(launches_per_apply + (1 if k == 1 and info["n_hot"] > 0 else 0) for k in ks)
-    # per PageRank call: init, scale, reduce, then per iteration the hot-row
-    # packing, the task kernel, the combine pass (if rows are split), the
-    # update and the reduce
-    launches_per_pr_iter = (3 + (1 if info["n_split_rows_t"] > 0 else 0)
-                            + (1 if info["n_hot_t"] > 0 else 0))
+    # per product: the task kernel and, if rows are split, the combine pass (part
+    # of the task kernel on lists of at most 16384 tasks, except with hot rows)
+    def launches_per_apply(k, suffix=""):
+        hot = k == 1 and info["n_hot" + suffix] > 0
+        return 1 + (1 if info["n_split_rows" + suffix] > 0 and (hot or info["n_tasks" + suffix] > 16384) else 0)
+    sweep_launches = sum(launches_per_apply(k) for k in ks)
+    # per PageRank call: init, scale, reduce, then per iteration the product and the update
+    launches_per_pr_iter = launches_per_apply(1, "_t") + 1
     xpr = torch.empty(N, dtype=torch.float32, device=dev)
     pr_res = [None]
 
@@ -1141,7 +1139,7 @@ def main():
     # The dominant kernel: the task kernel's k = 1 instantiation (the k = 1
     # product of the sweep and the A^T product of every PageRank iteration,
     # 1 + iters launches per step), timed by the events around the sweep's
-    # k = 1 call (which also holds the hot-row copy and the split-row combine);
+    # k = 1 call (which also holds the split-row combine);
     # otherwise the slowest k of the sweep.
     kdom = 1 if (1 in ks and args.pagerank_iters) else max(ks, key=lambda k: statistics.median(per_k[k]))
     dom = breakdown[str(kdom)]
