@@ -163,20 +163,23 @@ def _ptr(a) -> _P:
 _DTYPE_CODES: dict = {}
 _raw_stream = None
 _F32 = None
+_Tensor = None
 
 
 def _load_torch():
-    global _raw_stream, _F32
+    global _raw_stream, _F32, _Tensor, _DTYPE_CODES
     import torch
     _F32 = torch.float32
-    _DTYPE_CODES.update({torch.float32: SPMM_F32, torch.bfloat16: SPMM_BF16, torch.float16: SPMM_F16,
-                         torch.float64: SPMM_F64})
+    _Tensor = torch.Tensor
     get = getattr(torch._C, "_cuda_getCurrentRawStream", None)
     if get is None:
         _raw_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
     else:
         device = torch.cuda.current_device
         _raw_stream = lambda: get(device())  # noqa: E731
+    # last and whole: another thread that sees it finds the rest
+    _DTYPE_CODES = {torch.float32: SPMM_F32, torch.bfloat16: SPMM_BF16, torch.float16: SPMM_F16,
+                    torch.float64: SPMM_F64}
 
 
 def _torch_dtype_code(t) -> int:
@@ -641,7 +644,12 @@ class SparseMatrix:
         xtype = _torch_dtype_code(X)
         k = shape[1]
         if Y is None:
-            Y = X.new_empty((self.n_cols if transpose else self.n_rows, k), dtype=_F32)
+            out_rows = self.n_cols if transpose else self.n_rows
+            if type(X) is _Tensor:
+                Y = X.new_empty((out_rows, k), dtype=_F32)
+            else:                               # a subclass's new_empty would make one of its own kind
+                import torch
+                Y = torch.empty((out_rows, k), dtype=_F32, device=X.device)
             ldy = k
         else:
             if Y.dim() != 2 or Y.stride(1) != 1 or Y.dtype != _F32:

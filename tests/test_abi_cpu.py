@@ -112,3 +112,28 @@ def test_binding_structs_match_the_header(tmp_path):
         for field, _ in cls._fields_:
             f = getattr(cls, field)
             assert c[(name, field)] == (f.offset, f.size), (name, field)
+
+
+def test_product_output_is_a_plain_tensor():
+    """apply()'s result is a plain float32 tensor whatever kind of tensor X is
+    (the C call is stood in for: only the binding runs)."""
+    import torch
+    from paper_1602_02864_gb300 import spmm
+
+    class Sub(torch.Tensor):
+        pass
+
+    class Handle:
+        handle, n_rows, n_cols = 1, 5, 7
+
+    seen = []
+
+    def call(*args):
+        seen.append(args)
+        return 0
+
+    X = torch.zeros(7, 3, dtype=torch.bfloat16)
+    for x in (X, X.as_subclass(Sub), torch.nn.Parameter(X)):
+        Y = spmm.SparseMatrix._product(Handle, call, x, False, None, 0)
+        assert type(Y) is torch.Tensor and Y.shape == (5, 3) and Y.dtype == torch.float32 and not Y.requires_grad
+        assert seen[-1] == (1, X.data_ptr(), 3, 3, spmm.SPMM_BF16, Y.data_ptr(), 3, spmm.SPMM_F32, 0, 0)
