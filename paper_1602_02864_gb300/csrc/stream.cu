@@ -116,21 +116,8 @@ int stream_setup(spmm_mat* A, const int64_t* row_ptr, const int32_t* col_idx, co
         return cuda_fail(e, "streaming: pin row_ptr");
     if ((e = pin(col_idx, (size_t)nnz * 4, &S.reg_ci)) != cudaSuccess) return cuda_fail(e, "streaming: pin col_idx");
     if ((e = pin(values, (size_t)nnz * vsize, &S.reg_val)) != cudaSuccess) return cuda_fail(e, "streaming: pin values");
-    // the row pointers stay in HBM (padded as in the resident mode): a ninth of the
-    // bytes of a matrix of 16 entries a row, and one copy less per block (32 MB
-    // slots 1642 -> 1445 us).  Unless that memory is taken: then each block
-    // brings its own.
-    if (dmalloc((void**)&d.row_ptr, (size_t)(n + 3) * 8) == cudaSuccess) {
-        if ((e = cudaMemsetAsync(d.row_ptr + n + 1, 0, 16, s)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(d.row_ptr, row_ptr, (size_t)(n + 1) * 8, cudaMemcpyHostToDevice, s)) != cudaSuccess)
-            return cuda_fail(e, "streaming: row pointers");
-    } else {
-        cudaGetLastError();
-        d.row_ptr = nullptr;
-    }
     for (int i = 0; i < 2; ++i) {
         if ((e = dmalloc((void**)&S.slot_col[i], (size_t)S.slot_nnz * 4)) != cudaSuccess ||
-            (!d.row_ptr && (e = dmalloc((void**)&S.slot_rp[i], (size_t)S.slot_rows * 8)) != cudaSuccess) ||
             (vsize > 0 && (e = dmalloc(&S.slot_val[i], (size_t)S.slot_nnz * vsize)) != cudaSuccess))
             return cuda_fail(e, "streaming: staging slots");
     }
@@ -171,6 +158,21 @@ int stream_setup(spmm_mat* A, const int64_t* row_ptr, const int32_t* col_idx, co
                 return cuda_fail(e, "streaming: partials");
             *bytes += (int64_t)d.n_slots * kSlotStride * sizeof(float);
         }
+    }
+    // the row pointers stay in HBM (padded as in the resident mode): a ninth of the
+    // bytes of a matrix of 16 entries a row, and one copy less per block (32 MB
+    // slots 1642 -> 1445 us).  Unless what the rest leaves free is too little:
+    // then each block brings its own.
+    if (dmalloc((void**)&d.row_ptr, (size_t)(n + 3) * 8) == cudaSuccess) {
+        if ((e = cudaMemsetAsync(d.row_ptr + n + 1, 0, 16, s)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(d.row_ptr, row_ptr, (size_t)(n + 1) * 8, cudaMemcpyHostToDevice, s)) != cudaSuccess)
+            return cuda_fail(e, "streaming: row pointers");
+    } else {
+        cudaGetLastError();
+        d.row_ptr = nullptr;
+        for (int i = 0; i < 2; ++i)
+            if ((e = dmalloc((void**)&S.slot_rp[i], (size_t)S.slot_rows * 8)) != cudaSuccess)
+                return cuda_fail(e, "streaming: staging slots");
     }
     S.bytes_per_apply = nnz * 4 + (int64_t)(nnz * vsize) + (d.row_ptr ? 0 : (n + 1) * 8);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "streaming: set-up");
