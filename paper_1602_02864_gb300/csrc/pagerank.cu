@@ -76,8 +76,11 @@ __global__ void pr_scale_kernel(const float* __restrict__ x, const float* __rest
 // A sum of floats as three floats, each holding what the one before rounded
 // away (Knuth's two-sum): 72 bits, so no less exact than an FP64 sum, on the
 // FP32 units (an FP64 addition and its conversion take 32 times as long here).
+// Terms above 2^100, infinities and NaN, which the floats could not carry, are
+// added in FP64 (pr_add).
 struct FloatSum {
     float s = 0.f, c = 0.f, d = 0.f;
+    double big = 0.0;
     static __device__ __forceinline__ float two_sum(float& a, float b) {
         const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
         const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
@@ -85,8 +88,20 @@ struct FloatSum {
         return e;
     }
     __device__ __forceinline__ void add(float v) { d = __fadd_rn(d, two_sum(c, two_sum(s, v))); }
-    __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)d); }
+    __device__ __forceinline__ double value() const { return big + ((double)s + ((double)c + (double)d)); }
 };
+
+// r and dg into the two sums.  One test for both, as a branch: a test in each
+// sum took 3 us of an iteration on 4.2 M vertices, this one nothing measurable.
+__device__ __forceinline__ void pr_add(FloatSum& res, FloatSum& dang, float r, float dg) {
+    if (__builtin_expect(r + fabsf(dg) <= 0x1p100f, 1)) {
+        res.add(r);
+        dang.add(dg);
+    } else {
+        res.big += (double)r;
+        dang.big += (double)dg;
+    }
+}
 
 // x' = (1-d)/N + d*D/N + d*y, with D the dangling mass of x (scal[0]);
 // partials of sum |x' - x| and of the dangling mass of x'; z' = x' / L; the last
@@ -121,8 +136,7 @@ pr_update_kernel(const float* __restrict__ y, float* __restrict__ x, const float
             r += pr_elem(y4.w, x4.w, v4.w, base, df, z4.w, dg);
             reinterpret_cast<float4*>(x)[i] = x4;
             reinterpret_cast<float4*>(z)[i] = z4;
-            res.add(r);
-            dang.add(dg);
+            pr_add(res, dang, r, dg);
         };
         const float4 *y_4 = reinterpret_cast<const float4*>(y), *v_4 = reinterpret_cast<const float4*>(inv);
         const float4* x_4 = reinterpret_cast<const float4*>(x);
@@ -138,10 +152,10 @@ pr_update_kernel(const float* __restrict__ y, float* __restrict__ x, const float
     }
     for (int64_t i = done_n + tid; i < n; i += stride) {   // tail (or unaligned buffers)
         float xi = x[i], zi, dg = 0.f;
-        res.add(pr_elem(y[i], xi, inv[i], base, df, zi, dg));
+        const float r = pr_elem(y[i], xi, inv[i], base, df, zi, dg);
         x[i] = xi;
         z[i] = zi;
-        dang.add(dg);
+        pr_add(res, dang, r, dg);
     }
     const double s1 = block_sum(res.value(), sh);
     const double s2 = block_sum(dang.value(), sh);

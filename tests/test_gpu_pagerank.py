@@ -134,3 +134,20 @@ def test_pagerank_cached_graph_follows_its_inputs(sp):
         h.sync_status()
     finally:
         h.close()
+
+
+def test_residual_of_huge_and_infinite_ranks(sp):
+    """The L1 change of ranks near the largest float32 (a thread's terms exceed it in
+    sum) and of an infinite one.  On a cycle with every rank 3e38 and damping 0.85
+    each term is |0.85 * 3e38 - 3e38| = 4.5e37; the float32 roundings of 0.85, the
+    product and the sums of four terms are below 2e-6 of it."""
+    import torch
+    n = 1 << 20
+    h = handle(sp, graphs.cycle(n))
+    x, res = h.pagerank(0.85, 1, x0=torch.full((n,), 3e38, device="cuda"))
+    np.testing.assert_allclose(res, [n * 4.5e37], rtol=2e-6)
+    x0 = torch.full((n,), 1.0 / n, device="cuda")
+    x0[12345] = float("inf")       # its successor becomes infinite, itself finite: both changes are infinite
+    x, res = h.pagerank(0.85, 1, x0=x0)
+    assert np.isposinf(res[0]) and int(torch.isinf(x).sum()) == 1
+    h.close()
