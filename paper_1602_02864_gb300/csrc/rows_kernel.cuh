@@ -341,6 +341,14 @@ constexpr int min_blocks() {
     return (MG == 2 && VMODE == 0) ? 4 : two_blocks<VMODE, CH, ONE, MG>() ? 2 : SPMM_MIN_BLOCKS;
 }
 
+// *p counted up, wrapping to zero after `last`; everything before it is visible
+// to whoever sees the new count and then fences.
+__device__ __forceinline__ unsigned int atom_inc_release(unsigned int* p, unsigned int last) {
+    unsigned int old;
+    asm volatile("atom.inc.release.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(last) : "memory");
+    return old;
+}
+
 // A segment of a split row has its partial in a.partials: returns the row's
 // split if this was its last segment to arrive, -1 otherwise.  The arrival is a
 // release, not a full fence, which would empty L1 as well.
@@ -349,11 +357,7 @@ __device__ __forceinline__ int segment_done(const FwdArgs& a, int slot, int lane
     const int2 seg = a.slot_seg[slot];     // {split, segments of its row}
     __syncwarp();                          // the lanes' parts of the partial, before the arrival
     unsigned int before = 0;
-    if (lane == 0)                         // wraps to zero at the last arrival
-        asm volatile("atom.inc.release.gpu.global.u32 %0, [%1], %2;"
-                     : "=r"(before)
-                     : "l"(a.seg_done + seg.x), "r"((unsigned int)seg.y - 1u)
-                     : "memory");
+    if (lane == 0) before = atom_inc_release(a.seg_done + seg.x, (unsigned int)seg.y - 1u);   // zero at the last
     return (int)__shfl_sync(0xffffffffu, before, 0) + 1 == seg.y ? seg.x : -1;
 }
 
@@ -1111,7 +1115,10 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
             }
         }
         if (SEG && ready >= 0) {   // add its segments' partials, in segment order, into Y
-            __threadfence();    // the other warps' partials, after their arrivals
+            // lane 0 saw the other warps' arrivals: its fence, then the warp's barrier, put every
+            // lane's reads of their partials after them
+            __threadfence();
+            __syncwarp();
             const FwdArgs& a = *cur;
             combine_row(a.splits[ready], a.partials, a.Y, a.ldy, a.k, combine_lanes_log2(a.k), a.partials_comp, lane);
         }
@@ -1127,15 +1134,20 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
 
 // The end of a warp: the launch's last one leaves the task counter at zero for
 // the next launch.  After a wait that ran out (in this launch or one not yet
-// reported) some segments may be missing, so it clears the arrivals too.
+// reported) some segments may be missing, so it clears the arrivals too.  Every
+// warp's arrival here is a release and the last one's is followed by a fence, so
+// the last warp sees each status bit, claim and segment arrival of the launch
+// before it reads or clears them.
 __device__ __forceinline__ void warp_done(const FwdArgs& ga, const MultiArgs* M) {
     if (!ga.ctl) return;
     __syncwarp();
     const int lane = threadIdx.x & 31;
     const unsigned int warps = gridDim.x * (blockDim.x >> 5);
     unsigned int old = 0;
-    if (lane == 0) old = atomicInc(&ga.ctl->done, warps - 1);    // wraps to zero at the last
+    if (lane == 0) old = atom_inc_release(&ga.ctl->done, warps - 1);    // wraps to zero at the last
     if (__shfl_sync(0xffffffffu, old, 0) != warps - 1) return;
+    __threadfence();
+    __syncwarp();
     if (lane == 0) ga.ctl->next = 0;
     if (__ldcg(ga.status) == 0) return;
     for (int e = 0; e < (M ? M->n : 1); ++e) {
