@@ -55,6 +55,12 @@ struct TaskCtl {
     unsigned int next, done, cleared_next, pad;
 };
 
+// Entries from e0 to e1, at most 2^31 - 1 of them, by the low words of both: the
+// difference wraps where an odd multiple of 2^31 lies between.
+__host__ __device__ constexpr int entries_between(int e0_low, int e1_low) {
+    return (int)((uint32_t)e1_low - (uint32_t)e0_low);
+}
+
 struct HostPlan {
     std::vector<int4> tasks;    // n_tasks + 1 (sentinel)
     std::vector<int4> splits;

@@ -256,7 +256,7 @@ struct Staged {
     int e0;                     // low word of the task's first nonzero
     // start of row j among the task's nonzeros (the low words' difference)
     __device__ __forceinline__ int rp(int j) const {
-        return (int)(reinterpret_cast<const uint32_t*>(rpw)[2 * j] - (uint32_t)e0);
+        return entries_between(e0, (int)reinterpret_cast<const uint32_t*>(rpw)[2 * j]);
     }
 };
 
@@ -547,7 +547,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     auto take = [&](const Desc& x) {
         d0 = make_int2(x.a.x, x.a.y);
         e0 = x.a.z;
-        n = x.end.x - e0;
+        n = entries_between(e0, x.end.x);
     };
     take(nx);
     // the next task: static stride, or the next of a chunk claimed from the

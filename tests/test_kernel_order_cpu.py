@@ -45,3 +45,20 @@ def test_combining_warp_reads_partials_after_their_arrivals():
     src = kernel_source()
     in_order(body(src, "int segment_done("), "__syncwarp();", "atom_inc_release(a.seg_done")
     in_order(src[src.index("ready >= 0"):], "__threadfence();", "__syncwarp();", "combine_row(")
+
+
+def test_task_length_across_two_to_the_31(tmp_path):
+    """The length of a task from the low words of its ends, where an odd multiple of 2^31
+    nonzeros lies between them: evaluated as a constant, in which a signed overflow is an error."""
+    import subprocess
+    from paper_1602_02864_gb300 import build
+    src = tmp_path / "len.cu"
+    src.write_text('#include "internal.h"\n'
+                   "using spmm::entries_between;\n"
+                   "constexpr int top = 0x7fffff00, low = -0x7fffff00;\n"
+                   'static_assert(entries_between(top, low) == 512, "across 2^31");\n'
+                   'static_assert(entries_between(-256, 256) == 512, "across 2^32");\n'
+                   'static_assert(entries_between(5, 5) == 0 && entries_between(5, 517) == 512, "plain");\n')
+    subprocess.check_call([build.nvcc(), *build.ARCH, *build.NVCC_FLAGS, "-c", str(src), "-o", str(tmp_path / "len.o")])
+    src = kernel_source()
+    assert "n = entries_between(e0, x.end.x)" in src and "x.end.x - e0" not in src
