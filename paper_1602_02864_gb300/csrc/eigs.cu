@@ -260,33 +260,18 @@ __global__ void f32_to_bf16_kernel(const float* __restrict__ src, int64_t total,
         dst[t] = __float2bfloat16(src[t]);
 }
 
-// 1 / sqrt(d) for a positive normal d: the FP32 value of d scaled by a power of
-// four to [1, 4), refined twice (y += y (1 - d y^2) / 2; relative error 1e-7,
-// 1e-14, then the rounding of the last step).
-__device__ __forceinline__ double rsqrt_newton(double d) {
-    const int hi = __double2hiint(d), e = ((hi >> 20) - 1023) & ~1;
-    const double m = __hiloint2double(hi - (e << 20), __double2loint(d));
-    double y = (double)rsqrtf((float)m);
-    const double half = 0.5 * m;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const double r = fma(-half * y, y, 0.5);
-        y = fma(y, r, y);
-    }
-    return __hiloint2double(__double2hiint(y) - ((e / 2) << 20), __double2loint(y));
-}
-
 // Block Cholesky G = R^T R (R upper, b x b row-major, b <= B <= 32) and its
 // inverse Rinv = R^-1 (upper), by one warp: lane i holds column i in registers,
 // a pivot's row is passed by shuffles and its multiples are subtracted from the
 // rows below (the same differences in the same order as the left-looking
 // form); then lane c builds column c of the inverse by back substitution, row
-// by row.  Bound by its FP64 instructions, 64 clocks each on one scheduler, so
-// a pivot costs one reciprocal square root (FP32 and two Newton steps) instead
-// of a square root and two divisions (b = 16: 41 -> 23 us).  A pivot that is not
-// safely positive (below 1e-24 x trace) marks *flag and leaves the identity in
-// Rinv, so the kernels queued after it keep running on finite numbers until the
-// host reads the flag.
+// by row.  Bound by its FP64 instructions, 64 clocks each on one scheduler, in a
+// chain through the pivots.  Square roots and divisions are correctly rounded: a
+// reciprocal square root refined from FP32 takes 23 us instead of 44 (b = 16, 10
+// launches a restart) but is off by an ulp or two, and by far more at a subnormal
+// pivot.  A pivot that is not safely positive (below 1e-24 x trace) marks *flag and
+// leaves the identity in Rinv, so the kernels queued after it keep running on
+// finite numbers until the host reads the flag.
 template <int B>
 __global__ void __launch_bounds__(32) chol_inv_kernel(const double* __restrict__ G, int b, double* __restrict__ Rinv,
                                                       int32_t* __restrict__ flag) {
@@ -298,7 +283,7 @@ __global__ void __launch_bounds__(32) chol_inv_kernel(const double* __restrict__
     const double floor_d = 1e-24 * (tr > 0 ? tr : 1.0);
 #pragma unroll
     for (int k = 0; k < B; ++k) a[k] = (t < b && k <= t) ? G[k * b + t] : 0.0;
-    double rdiag = 1.0;                          // 1 / R[t][t]
+    double rdiag = 1.0;                          // R[t][t]
     bool bad = false;
 #pragma unroll
     for (int j = 0; j < B; ++j) {
@@ -306,9 +291,10 @@ __global__ void __launch_bounds__(32) chol_inv_kernel(const double* __restrict__
             const double d = __shfl_sync(0xffffffffu, a[j], j);
             bad = !(d > floor_d);
             if (!bad) {
-                const double y = rsqrt_newton(d);
-                a[j] *= y;                       // lane j: sqrt(d)
-                if (t == j) rdiag = y;
+                double r = 0.0;                  // on the lanes that need it only: FP64 takes as long as its lanes
+                if (t == j) a[j] = rdiag = r = sqrt(d);
+                r = __shfl_sync(0xffffffffu, r, j);
+                if (t > j && t < b) a[j] /= r;
                 if (t < b) R[j * B + t] = t >= j ? a[j] : 0.0;
 #pragma unroll
                 for (int k = j + 1; k < B; ++k)
@@ -338,11 +324,16 @@ __global__ void __launch_bounds__(32) chol_inv_kernel(const double* __restrict__
                     else s0 = fma(R[i * B + k], x[k], s0);
                 }
             const double ri = __shfl_sync(0xffffffffu, rdiag, i);
-            if (i == t) x[i] = ri;
-            else if (i < t) x[i] = -(s0 + s1) * ri;
+            if (i <= t && t < b) x[i] = (i == t ? 1.0 : -(s0 + s1)) / ri;
             if (t < b) Rinv[i * b + t] = x[i];
         }
     }
+}
+
+cudaError_t chol_inverse(const double* G, int b, double* Rinv, int32_t* flag, cudaStream_t s) {
+    if (b <= 16) chol_inv_kernel<16><<<1, 32, 0, s>>>(G, b, Rinv, flag);
+    else chol_inv_kernel<32><<<1, 32, 0, s>>>(G, b, Rinv, flag);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- host linear algebra
@@ -515,8 +506,7 @@ struct Eig {
         }
         for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
             if ((e = ts_tn(W, b, b, W, b, b, n, part, small, s)) != cudaSuccess) break;
-            if (b <= 16) chol_inv_kernel<16><<<1, 32, 0, s>>>(small, b, small2, flags + slot);
-            else chol_inv_kernel<32><<<1, 32, 0, s>>>(small, b, small2, flags + slot);
+            if ((e = chol_inverse(small, b, small2, flags + slot, s)) != cudaSuccess) break;
             e = ts_nn(W, b, b, small2, b, W2, b, n, 1.0, 0.0, s);
             std::swap(W, W2);
         }

@@ -1,4 +1,4 @@
-// tallskinny.h -- FP64 products of tall, narrow matrices (tallskinny.cu).
+// tallskinny.h -- FP64 products of tall, narrow matrices (tallskinny.cu) and the Cholesky factor of a Gram matrix.
 #pragma once
 
 #include "internal.h"
@@ -17,5 +17,9 @@ cudaError_t ts_nn(const double* A, int64_t lda, int p, const double* C, int q, d
 // the column norms squared of R = AU - U diag(theta) (n x q, contiguous): out[j] = sum_i R[i][j]^2
 cudaError_t ts_residuals(const double* AU, const double* U, const double* theta, int q, int64_t n, double* partial,
                          double* out, cudaStream_t s);
+
+// Rinv (b x b, upper) = R^-1 of the Cholesky factor G = R^T R, b <= 32 (eigs.cu); *flag = 1 and the identity
+// where a pivot is not safely positive
+cudaError_t chol_inverse(const double* G, int b, double* Rinv, int32_t* flag, cudaStream_t s);
 
 }  // namespace spmm

@@ -52,6 +52,13 @@ int spmm_probe_ts_tn(const double* A, int64_t lda, int32_t p, const double* B, i
 int spmm_probe_ts_nn(const double* A, int64_t lda, int32_t p, const double* C, int32_t q, double* Out, int64_t ldo,
                      int64_t n, double alpha, double beta, void* stream);
 
+/*
+ * spmm_probe_chol_inv -- diagnostic: Rinv (b x b, row-major, upper) = R^-1 of
+ * G = R^T R (device arrays, 1 <= b <= 32) as the eigensolvers form it; *flag
+ * (device) becomes 1 where a pivot is not safely positive.  Synchronises `stream`.
+ */
+int spmm_probe_chol_inv(const double* G, int32_t b, double* Rinv, int32_t* flag, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

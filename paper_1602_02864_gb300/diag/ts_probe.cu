@@ -31,3 +31,14 @@ extern "C" int spmm_probe_ts_nn(const double* A, int64_t lda, int32_t p, const d
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     return e == cudaSuccess ? SPMM_OK : cuda_fail(e, "spmm_probe_ts_nn");
 }
+
+extern "C" int spmm_probe_chol_inv(const double* G, int32_t b, double* Rinv, int32_t* flag, void* stream) {
+    if (!G || !Rinv || !flag || b < 1 || b > 32) {
+        set_error("spmm_probe_chol_inv: need non-NULL arrays and 1 <= b <= 32");
+        return SPMM_ERR_ARG;
+    }
+    cudaStream_t s = (cudaStream_t)stream;
+    cudaError_t e = chol_inverse(G, b, Rinv, flag, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e == cudaSuccess ? SPMM_OK : cuda_fail(e, "spmm_probe_chol_inv");
+}

@@ -23,6 +23,8 @@ _lib.spmm_probe_ts_tn.argtypes = [_P, _i64, _i32, _P, _i64, _i32, _i64, _P, _P]
 _lib.spmm_probe_ts_tn.restype = ctypes.c_int
 _lib.spmm_probe_ts_nn.argtypes = [_P, _i64, _i32, _P, _i32, _P, _i64, _i64, ctypes.c_double, ctypes.c_double, _P]
 _lib.spmm_probe_ts_nn.restype = ctypes.c_int
+_lib.spmm_probe_chol_inv.argtypes = [_P, _i32, _P, _P, _P]
+_lib.spmm_probe_chol_inv.restype = ctypes.c_int
 
 
 def spmm_probe_gather(table_bytes, row_bytes, stream=None):
@@ -55,3 +57,10 @@ def spmm_probe_ts_nn(A, C, Out, alpha, beta, stream=None):
                                      Out.stride(0), A.shape[0], float(alpha), float(beta),
                                      _sp._stream_handle(stream)))
     return Out
+
+
+def spmm_probe_chol_inv(G, Rinv, flag, stream=None):
+    """Rinv = R^-1 of G = R^T R (float64 CUDA tensors, b x b); flag: an int32 CUDA tensor."""
+    _sp._check(_lib.spmm_probe_chol_inv(_sp._ptr(G), G.shape[0], _sp._ptr(Rinv), _sp._ptr(flag),
+                                        _sp._stream_handle(stream)))
+    return Rinv
