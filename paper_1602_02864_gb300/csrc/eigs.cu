@@ -16,7 +16,7 @@
 // are the residuals).
 //
 // The Krylov-Schur solver's tall-skinny FP64 products, C = A^T B and
-// Out = beta Out + alpha A C, are in tallskinny.cu.
+// Out = beta Out + alpha A C, are in tallskinny.cu (but for W R^-1: nn_upper).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -32,8 +32,8 @@ constexpr int kEigThreads = 256;
 constexpr int kEigMaxBasis = 64;
 constexpr int kTsTile = 16;
 
-// ---- the same products in FP64 arithmetic, for the filtered iteration.  A
-// filter of degree 20 multiplies the block's trailing directions' rounding by
+// ---- the same products in FP64 arithmetic, for the filtered iteration (and
+// W R^-1 of both solvers).  A filter of degree 20 multiplies the block's trailing directions' rounding by
 // its own amplification, so there the sums keep their order: products rounded
 // differently in the last place give eigenvectors 1e-4 apart before
 // convergence.  Bound by the FP64 units (two fused multiply-adds per clock and
@@ -448,17 +448,24 @@ struct Eig {
         }
         return download(p * q, out, e);
     }
+    // Out = A C with C upper triangular (q x q), A and Out contiguous.  FP64
+    // arithmetic in both solvers: C is R^-1 of a nearly orthonormal block, near the
+    // identity, so an element of Out is one element of A, often far below its row's
+    // largest, and 3-14% of them are below the line of ts_nn (tallskinny.cu).
+    static size_t upper_smem(int q) { return ((size_t)q * q + 64 * (size_t)(q | 1)) * sizeof(double); }
+    static bool fits_upper(int q) { return upper_smem(q) <= 48 * 1024; }
+    cudaError_t nn_upper(const double* Am, const double* C, int q, double* Out) {
+        plain_nn_upper_kernel<<<grid, kEigThreads, upper_smem(q), s>>>(Am, C, q, Out, n);
+        return cudaGetLastError();
+    }
     // Out = A C (C from the host; upper: C is upper triangular and A, Out are contiguous)
     cudaError_t nn(const double* Am, int64_t lda, int p, const std::vector<double>& C, int q, double* Out, int64_t ldo,
                    bool upper = false) {
         cudaError_t e = cudaMemcpyAsync(small, C.data(), (size_t)p * q * sizeof(double), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess && !plain) e = ts_nn(Am, lda, p, small, q, Out, ldo, n, 1.0, 0.0, s);
-        if (e == cudaSuccess && plain) {
-            const size_t smem = ((size_t)q * q + 64 * (size_t)(q | 1)) * sizeof(double);
-            if (upper && smem <= 48 * 1024)
-                plain_nn_upper_kernel<<<grid, kEigThreads, smem, s>>>(Am, small, q, Out, n);
-            else
-                plain_nn_kernel<<<grid, kEigThreads, 0, s>>>(Am, lda, p, small, q, Out, ldo, n);
+        if (e == cudaSuccess) {
+            if (upper && fits_upper(q)) e = nn_upper(Am, small, q, Out);
+            else if (!plain) e = ts_nn(Am, lda, p, small, q, Out, ldo, n, 1.0, 0.0, s);
+            else plain_nn_kernel<<<grid, kEigThreads, 0, s>>>(Am, lda, p, small, q, Out, ldo, n);
         }
         // small is reused by the next call: finish this one first
         return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
@@ -507,7 +514,7 @@ struct Eig {
         for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
             if ((e = ts_tn(W, b, b, W, b, b, n, part, small, s)) != cudaSuccess) break;
             if ((e = chol_inverse(small, b, small2, flags + slot, s)) != cudaSuccess) break;
-            e = ts_nn(W, b, b, small2, b, W2, b, n, 1.0, 0.0, s);
+            e = nn_upper(W, small2, b, W2);      // b <= 32 always fits
             std::swap(W, W2);
         }
         return e;

@@ -23,12 +23,25 @@
 //     FP64 (one FP64 addition per element and tile instead of kTsRows fused
 //     multiply-adds).
 // What is left out (i + j >= 8, and bits below 2^-62 of the largest element) is
-// at most 2^-59 of the product of the two scales per term, and usually far
-// below the rounding of an FP64 sum.  Largest error against quadruple
-// precision, FP64 kernels -> these: A^T B, 20,000 x 48 by 16, orthonormal columns
-// 7.7e-18 -> 4.9e-18, with rows of very different size 4.9e-16 -> 2.0e-16,
-// power-law rows 3.3e-16 -> 6.9e-17; A C, 2-norm of the error, 4.6e-17 -> 9.3e-18,
-// 8.7e-16 -> 1.6e-16, 5.1e-16 -> 8.6e-17.
+// at most 2^-58.8 of the product of the two scales per term.  By itself that is a
+// bound on the norm: where the large elements of the two operands do not meet, an
+// FP64 sum is far more accurate (one element of 1 among 1e-8 in each column, in
+// different rows: 1e-12 of sum |a||b| against 2e-17).  So every element's sum of
+// |a||b| is found from below as well (magnitudes cut to bf16, one mma beside the
+// 36), and an element whose sum is below 2^-5 of the scales' product takes the
+// products in FP64 arithmetic instead.  Above that line what is left out is less
+// than kTsRows * 2^-53 * sum |a||b| (0.6 of it), the bound of an FP64 sum of as
+// many products: the error bound of each element is that of FP64 arithmetic,
+// whatever the data.  FP64 arithmetic also takes the elements whose columns (rows)
+// hold subnormal numbers or whose scales are near the ends of the exponent range.
+// Share of the elements below the line, block Krylov-Schur on a symmetrised R-MAT
+// graph: A^T B 0.01%, the subtraction of V C 3%, Ritz vectors none; W R^-1 would
+// have 3-14%, and stays in FP64 arithmetic (eigs.cu).
+// A tile (row) with an infinity or a NaN gives NaN.
+// Largest error against quadruple precision, FP64 kernels -> digits: A^T B,
+// 20,000 x 48 by 16, orthonormal columns 7.7e-18 -> 4.9e-18, with rows of very
+// different size 4.9e-16 -> 2.0e-16, power-law rows 3.3e-16 -> 6.9e-17; A C, 2-norm
+// of the error, 4.6e-17 -> 9.3e-18, 8.7e-16 -> 1.6e-16, 5.1e-16 -> 8.6e-17.
 // Digits are made with integer instructions only, since conversions to and from
 // FP64 run at the rate of the FP64 units.  Measured, one restart of the block
 // Krylov-Schur solver on 148,444 vertices (basis 64, block 16; 26 products of each
@@ -50,13 +63,46 @@ constexpr int kTsRows = 64;          // rows per tile of ts_tn: diagonal sums st
 constexpr int kTsWarps = 12;         // warps per block, one block per SM (at most 168 registers a thread)
 constexpr int kDigits = 8;
 
-// The largest magnitude of a set is kept as its high word without the sign,
-// its biased exponent as kSpecial where an infinity or a NaN is among it.
+// A magnitude is kept as its high word without the sign, the last bit set where
+// the low word is not zero: 0 for a zero only.  The largest of a set gives its
+// biased exponent: kNoExp where all are zero, kSpecial where an infinity or a NaN
+// is among them.
 constexpr int kSpecial = 1 << 20;
-__device__ __forceinline__ int exponent_of(uint32_t hi) { return (hi >> 20) >= 0x7ffu ? kSpecial : (int)(hi >> 20); }
-__device__ __forceinline__ uint32_t hi_abs(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
+constexpr int kNoExp = -100000;
+__device__ __forceinline__ uint32_t magnitude(uint32_t lo, uint32_t hi) { return (hi & 0x7fffffffu) | min(lo, 1u); }
+__device__ __forceinline__ uint32_t magnitude(double x) {
+    return magnitude((uint32_t)__double2loint(x), (uint32_t)__double2hiint(x));
+}
+__device__ __forceinline__ uint32_t magnitude_at(const double* p) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    return magnitude(v.x, v.y);
+}
+__device__ __forceinline__ int exponent_of(uint32_t h) {
+    return h == 0 ? kNoExp : (h >> 20) >= 0x7ffu ? kSpecial : (int)(h >> 20);
+}
 
-__device__ __forceinline__ uint32_t high_word(const double* p) { return __ldg(reinterpret_cast<const uint32_t*>(p) + 1); }
+// A magnitude over its set's scale 2^(emax - 1022), cut to a bf16 (so not above
+// it), as a bf16 pair; below 2^-125 zero.
+__device__ __forceinline__ uint32_t bf16_below(uint32_t h, int emax) {
+    const int de = emax - (int)(h >> 20);
+    return (uint32_t)de < 125u ? (uint32_t)(126 - de) << 7 | ((h >> 13) & 0x7fu) : 0u;
+}
+__device__ __forceinline__ uint32_t bf16_pair(uint32_t h0, uint32_t h1, int e0, int e1) {
+    return bf16_below(h0, e0) | bf16_below(h1, e1) << 16;
+}
+
+// Whether an element with scales 2^(ea - 1022), 2^(eb - 1022) and at least `low`
+// of their product as its sum of |a||b| takes FP64 arithmetic: below the line, with
+// subnormal elements that count (sub), or with a result that could leave the normal
+// numbers.  Products with a zero set are exact, those with an infinity or a NaN are
+// NaN.
+constexpr float kLowLine = 0x1p-5f;
+__device__ __forceinline__ bool needs_fp64(float low, int ea, int eb, bool sub) {
+    if (max(ea, eb) >= kSpecial) return false;
+    if (sub) return true;
+    if (min(ea, eb) < -50000) return false;
+    return !(low >= kLowLine) || ea + eb < 1090 || ea + eb > 3061;
+}
 
 // x as eight digits + 128, most significant in the top byte: the 62-bit fixed
 // point of x / 2^(emax - 1022), truncated towards zero, plus 0x80 in every byte.
@@ -94,6 +140,14 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], u
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
 // all digits of one operand fragment: four (A) or two (B) registers per digit
 template <int I>
 __device__ __forceinline__ void a_digits(uint32_t (&f)[kDigits][4], const uint2 (&y)[8]) {
@@ -123,7 +177,8 @@ __device__ __forceinline__ void mma_digits(float (&acc)[kDigits][4], const uint3
 }
 
 // sum_d S_d 2^(56 - 8d) * 2^(ea + eb - 2112), rounded once to FP64: the value
-// of one element from its eight diagonals and the two biased exponents.
+// of one element from its eight diagonals and the two biased exponents (a normal
+// number or zero unless needs_fp64).
 __device__ __forceinline__ double from_diagonals(const float (&acc)[kDigits][4], int c, int ea, int eb) {
     int64_t h = 0, l = 0;
 #pragma unroll
@@ -152,9 +207,7 @@ __device__ __forceinline__ double from_diagonals(const float (&acc)[kDigits][4],
         int be = 1023 + 95 - lz + e2;            // biased exponent of m * 2^(32 - lz + e2)
         const uint64_t q = m + 1024u;            // round to nearest at bit 11
         if (q < m) ++be;                         // carried out: the mantissa is 1.0
-        uint64_t bits = (uint64_t)be << 52 | (q < m ? 0ull : (q >> 11) & 0xfffffffffffffull);
-        if (be <= 0) bits = 0;
-        if (be >= 2047) bits = 0x7ff0000000000000ull;
+        const uint64_t bits = (uint64_t)be << 52 | (q < m ? 0ull : (q >> 11) & 0xfffffffffffffull);
         r = __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
     }
     // a set with an infinity or a NaN
@@ -163,8 +216,8 @@ __device__ __forceinline__ double from_diagonals(const float (&acc)[kDigits][4],
 
 // Warp w of the launch owns unit w % units (16 columns of A by 16 of B) and the
 // row tiles w / units, + kgroups, ...; no shared memory and no barriers: a
-// tile's column scales are found in a first pass over its high words, which
-// also brings the tile into L1 for the second.  In a fragment, lane 4g + t
+// tile's column scales and the sums of its magnitudes are found in a first pass,
+// which also brings the tile into L1 for the second.  In a fragment, lane 4g + t
 // holds rows 2t, 2t+1, 2t+8, 2t+9 of a 16-row step and columns g, g+8.
 // SAME: A is B; units are the tile pairs of the upper triangle.
 template <bool SAME>
@@ -201,35 +254,67 @@ ts_tn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
         const int64_t r0 = tile * kTsRows;
         // row r of step ks; rows past the last repeat it (and count as zero in the products)
         auto row_of = [&](int ks, int r) { return min(r0 + ks * 16 + 2 * t + (r & 1) + (r >> 1) * 8, n - 1); };
-        uint32_t ha0 = 0, ha1 = 0, hb0 = 0, hb1 = 0;
+        uint32_t h[kTsRows / 16][4][4], hm[4] = {0, 0, 0, 0};     // A0, A1, B0, B1
 #pragma unroll
-        for (int ks = 0; ks < kTsRows / 16; ++ks) {
-            uint32_t h[4][4];
+        for (int ks = 0; ks < kTsRows / 16; ++ks)
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const int64_t ra = row_of(ks, r) * lda, rb = row_of(ks, r) * ldb;
-                h[0][r] = high_word(A0 + ra);
-                h[1][r] = high_word(A1 + ra);
-                h[2][r] = diag ? 0u : high_word(B0 + rb);
-                h[3][r] = diag ? 0u : high_word(B1 + rb);
+                h[ks][0][r] = magnitude_at(A0 + ra);
+                h[ks][1][r] = magnitude_at(A1 + ra);
+                h[ks][2][r] = diag ? 0u : magnitude_at(B0 + rb);
+                h[ks][3][r] = diag ? 0u : magnitude_at(B1 + rb);
             }
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                ha0 = max(ha0, h[0][r] & 0x7fffffffu);
-                ha1 = max(ha1, h[1][r] & 0x7fffffffu);
-                hb0 = max(hb0, h[2][r] & 0x7fffffffu);
-                hb1 = max(hb1, h[3][r] & 0x7fffffffu);
-            }
-        }
+        for (int i = 0; i < 4; ++i) {
 #pragma unroll
-        for (int off = 1; off < 4; off <<= 1) {
-            ha0 = max(ha0, __shfl_xor_sync(0xffffffffu, ha0, off));
-            ha1 = max(ha1, __shfl_xor_sync(0xffffffffu, ha1, off));
-            hb0 = max(hb0, __shfl_xor_sync(0xffffffffu, hb0, off));
-            hb1 = max(hb1, __shfl_xor_sync(0xffffffffu, hb1, off));
+            for (int ks = 0; ks < kTsRows / 16; ++ks)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) hm[i] = max(hm[i], h[ks][i][r]);
+#pragma unroll
+            for (int off = 1; off < 4; off <<= 1) hm[i] = max(hm[i], __shfl_xor_sync(0xffffffffu, hm[i], off));
         }
-        if (diag) hb0 = ha0, hb1 = ha1;
-        const int ea0 = exponent_of(ha0), ea1 = exponent_of(ha1), eb0 = exponent_of(hb0), eb1 = exponent_of(hb1);
+        if (diag) hm[2] = hm[0], hm[3] = hm[1];
+        const int ea0 = exponent_of(hm[0]), ea1 = exponent_of(hm[1]), eb0 = exponent_of(hm[2]), eb1 = exponent_of(hm[3]);
+        // bit 4j + c: element c of columns 8j.. takes FP64 arithmetic
+        uint32_t fp64 = 0;
+        {
+            float low[2][4];
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) low[j][c] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < kTsRows / 16; ++ks) {
+                uint32_t ua[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    uint32_t h0 = h[ks][i & 1][i & 2], h1 = h[ks][i & 1][(i & 2) + 1];
+                    if (r0 + ks * 16 + 2 * t + (i & 2) * 4 >= n) h0 = 0;
+                    if (r0 + ks * 16 + 2 * t + (i & 2) * 4 + 1 >= n) h1 = 0;
+                    ua[i] = bf16_pair(h0, h1, (i & 1) ? ea1 : ea0, (i & 1) ? ea1 : ea0);
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const uint32_t(&hb)[4] = h[ks][2 + j];
+                    const int eb = j ? eb1 : eb0;
+                    const uint32_t b0 = diag ? ua[j] : bf16_pair(hb[0], hb[1], eb, eb);
+                    const uint32_t b1 = diag ? ua[2 + j] : bf16_pair(hb[2], hb[3], eb, eb);
+                    mma_bf16(low[j], ua, b0, b1);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int eb = __shfl_sync(0xffffffffu, j ? eb1 : eb0, 4 * (2 * t + (c & 1)));
+                    const int ea = c < 2 ? ea0 : ea1;
+                    const bool inside = mi * 16 + g + (c < 2 ? 0 : 8) < p && ni * 16 + 8 * j + 2 * t + (c & 1) < q;
+                    // near the smallest normal numbers a subnormal element is not below the last digit
+                    const bool tiny = min(ea, eb) < 128 && min(ea, eb) >= 0;
+                    if (inside && needs_fp64(low[j][c], ea, eb, tiny)) fp64 |= 1u << (4 * j + c);
+                }
+        }
         float acc[2][kDigits][4];
 #pragma unroll
         for (int j = 0; j < 2; ++j)
@@ -290,8 +375,24 @@ ts_tn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int eb = __shfl_sync(0xffffffffu, j ? eb1 : eb0, 4 * (2 * t + (c & 1)));
-                sum[j][c] += from_diagonals(acc[j], c, c < 2 ? ea0 : ea1, eb);
+                if (!(fp64 >> (4 * j + c) & 1)) sum[j][c] += from_diagonals(acc[j], c, c < 2 ? ea0 : ea1, eb);
             }
+        if (__any_sync(0xffffffffu, fp64 != 0)) {
+            const int rows = (int)min((int64_t)kTsRows, n - r0);
+#pragma unroll 1
+            for (int e = 0; e < 8; ++e) {
+                double f = 0.0;
+                if (fp64 >> e & 1) {
+                    const double* a = ((e & 2) ? A1 : A0) + r0 * lda;
+                    const double* b = B + ni * 16 + 8 * (e >> 2) + 2 * t + (e & 1) + r0 * ldb;
+#pragma unroll 4
+                    for (int r = 0; r < rows; ++r) f = fma(a[r * lda], b[r * ldb], f);
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (u == e && (fp64 >> u & 1)) sum[u >> 2][u & 3] += f;
+            }
+        }
     }
     double* out = partial + (int64_t)kg * p * q;
 #pragma unroll
@@ -337,47 +438,60 @@ __global__ void __launch_bounds__(256) ts_reduce_kernel(const double* __restrict
 // in CholQR); then every column of C is scaled by its largest element.  The
 // digits of C sit in shared memory in fragment order (made once per block); a
 // warp takes 16 rows of A at a time and for each 16 columns of Out multiplies
-// the digits of up to 64 columns of A into one set of accumulators.
-constexpr int kNoExp = -100000;      // exponent of a zero
+// the digits of up to 64 columns of A into one set of accumulators.  With Out
+// added unscaled, an element of Out that is larger than what could be left out
+// times 2^53 hides it in the last rounding, and needs no FP64 arithmetic.
 __global__ void __launch_bounds__(kTsWarps * 32, 1)
 ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __restrict__ C, int q, double* Out,
              int64_t ldo, int64_t n, double alpha, double beta, int vec2) {
     extern __shared__ __align__(16) unsigned char ts_smem[];
     const int steps = (p + 15) >> 4, ntiles = (q + 7) >> 3;
     uint2* cd = reinterpret_cast<uint2*>(ts_smem);                                   // [ntile][step][digit][lane]
-    int* ce = reinterpret_cast<int*>(cd + (int64_t)ntiles * steps * kDigits * 32);   // exponent of column j of C
+    uint2* cb = cd + (int64_t)ntiles * steps * kDigits * 32;                         // [ntile][step][lane]: magnitudes
+    int* ce = reinterpret_cast<int*>(cb + (int64_t)ntiles * steps * 32);             // exponent of column j of C
     int* cr = ce + 64;                                                               // exponent of row k of C - 1023
     double* cs = reinterpret_cast<double*>(cr + 64);                                 // C
     for (int i = threadIdx.x; i < p * q; i += blockDim.x) cs[i] = C[i];
     __syncthreads();
+    bool sub = false;                                // a subnormal element of C
     for (int k = threadIdx.x; k < 64; k += blockDim.x) {
         uint32_t h = 0;
         if (k < p)
-            for (int j = 0; j < q; ++j) h = max(h, hi_abs(cs[k * q + j]));
+            for (int j = 0; j < q; ++j) {
+                const uint32_t x = magnitude(cs[k * q + j]);
+                h = max(h, x);
+                sub |= x != 0 && (x >> 20) == 0;
+            }
         cr[k] = (h >> 20) == 0 ? kNoExp : (int)(h >> 20) - 1023;
     }
-    __syncthreads();
+    const bool c_sub = __syncthreads_or(sub) != 0;
     for (int j = threadIdx.x; j < ntiles * 8; j += blockDim.x) {
         int e = 0;
-        bool special = false;
+        bool special = false, zero = true;
         if (j < q)
             for (int k = 0; k < p; ++k) {
-                const int x = (int)(hi_abs(cs[k * q + j]) >> 20);
+                const uint32_t h = magnitude(cs[k * q + j]);
+                const int x = (int)(h >> 20);
                 special |= x == 0x7ff;
+                zero &= h == 0;
                 if (x > 0) e = max(e, x - cr[k]);
             }
-        ce[j] = special ? kSpecial : e;
+        ce[j] = special ? kSpecial : zero ? kNoExp : e;
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     for (int f = warp; f < ntiles * steps; f += kTsWarps) {
         const int nt = f / steps, ks = f % steps, col = nt * 8 + g;
         uint2 y[4];
+        uint32_t m[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int k = ks * 16 + 2 * t + (r & 1) + (r >> 1) * 8;
-            y[r] = digits_of(k < p && col < q ? cs[k * q + col] : 0.0, ce[col] + cr[k]);
+            const double c = k < p && col < q ? cs[k * q + col] : 0.0;
+            y[r] = digits_of(c, ce[col] + cr[k]);
+            m[r] = bf16_below(magnitude(c), ce[col] + cr[k]);
         }
+        cb[f * 32 + lane] = make_uint2(m[0] | m[1] << 16, m[2] | m[3] << 16);
         uint32_t fb[kDigits][2];
         b_digits<0>(fb, y);
 #pragma unroll
@@ -385,6 +499,9 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
     }
     __syncthreads();
     const int64_t rtiles = (n + 15) >> 4;
+    // |Out| >= p 2^-4 of the scales' product: the last rounding is no less than what is left out
+    const bool hides = beta == 1.0 && (alpha == 1.0 || alpha == -1.0);
+    const int hidden = 1025 - (32 - __clz(p - 1));
     for (int64_t rt = (int64_t)blockIdx.x * kTsWarps + warp; rt < rtiles; rt += (int64_t)gridDim.x * kTsWarps) {
         const int64_t row0 = rt * 16 + g, row1 = row0 + 8;
         // rows past the last repeat it, columns past the last too (C's digits are zero there)
@@ -402,25 +519,62 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
                 for (int r = 0; r < 8; ++r) x[r] = ((r & 2) ? p1 : p0)[min(k + (r & 1) + (r >> 2) * 8, p - 1)];
             }
         };
-        int e0 = kNoExp, e1 = kNoExp;
+        int e0 = kNoExp, e1 = kNoExp, sub0 = 0, sub1 = 0;
+        uint32_t h[4][8];
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
+        for (int ks = 0; ks < 4; ++ks) {
             if (ks < steps) {
                 double x[8];
                 load8(ks, x);
 #pragma unroll
                 for (int r = 0; r < 8; ++r) {
                     const int k = ks * 16 + 2 * t + (r & 1) + (r >> 2) * 8;
-                    const int x20 = (int)(hi_abs(x[r]) >> 20);
-                    const int e = x20 == 0x7ff && k < p ? kSpecial : x20 == 0 ? kNoExp : x20 + cr[k];
-                    if (r & 2) e1 = max(e1, e);
-                    else e0 = max(e0, e);
+                    h[ks][r] = k < p ? magnitude(x[r]) : 0u;
+                    const int x20 = (int)(h[ks][r] >> 20);
+                    const int e = x20 == 0x7ff ? kSpecial : x20 == 0 ? kNoExp : x20 + cr[k];
+                    const int sb = x20 == 0 && h[ks][r] != 0;
+                    if (r & 2) e1 = max(e1, e), sub1 |= sb;
+                    else e0 = max(e0, e), sub0 |= sb;
                 }
             }
+        }
 #pragma unroll
         for (int off = 1; off < 4; off <<= 1) {
             e0 = max(e0, __shfl_xor_sync(0xffffffffu, e0, off));
             e1 = max(e1, __shfl_xor_sync(0xffffffffu, e1, off));
+            sub0 |= __shfl_xor_sync(0xffffffffu, sub0, off);
+            sub1 |= __shfl_xor_sync(0xffffffffu, sub1, off);
+        }
+        // bit 4 (tile of 8 columns) + c: that element takes FP64 arithmetic
+        uint32_t fp64 = 0;
+        {
+            uint32_t ua[4][4];
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+                if (ks < steps) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int* c = cr + ks * 16 + 2 * t + (i >> 1) * 8;
+                        const int e = (i & 1) ? e1 : e0;
+                        ua[ks][i] = bf16_pair(h[ks][2 * i], h[ks][2 * i + 1], e - c[0], e - c[1]);
+                    }
+                }
+            for (int nt = 0; nt < ntiles; ++nt) {
+                float low[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks)
+                    if (ks < steps) {
+                        const uint2 v = cb[(nt * steps + ks) * 32 + lane];
+                        mma_bf16(low, ua[ks], v.x, v.y);
+                    }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int col = nt * 8 + 2 * t + (c & 1), e = c < 2 ? e0 : e1;
+                    if (col < q && (c < 2 ? row0 : row1) < n &&
+                        needs_fp64(low[c], e, ce[col], c_sub || (c < 2 ? sub0 : sub1)))
+                        fp64 |= 1u << (4 * nt + c);
+                }
+            }
         }
         for (int np = 0; np < ntiles; np += 2) {
             float acc[2][kDigits][4];
@@ -464,9 +618,31 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
                         const int64_t row = min(c < 2 ? row0 : row1, n - 1);
                         o[c] = beta != 0.0 ? Out[row * ldo + min(col + (c & 1), q - 1)] : 0.0;
                     }
+                    uint32_t f64 = fp64 >> (4 * (np + j)) & 15u;
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        v[c] = from_diagonals(acc[j], c, c < 2 ? e0 : e1, ce[col + (c & 1)]);
+                        const int e = c < 2 ? e0 : e1, ec = ce[col + (c & 1)];
+                        v[c] = from_diagonals(acc[j], c, e, ec);
+                        if (hides && !c_sub && !(c < 2 ? sub0 : sub1) && (int)(magnitude(o[c]) >> 20) >= e + ec - hidden &&
+                            e + ec >= 1090 && e + ec <= 3061)
+                            f64 &= ~(1u << c);
+                    }
+                    if (__any_sync(0xffffffffu, f64 != 0)) {
+#pragma unroll 1
+                        for (int c = 0; c < 4; ++c) {
+                            double f = 0.0;
+                            if (f64 >> c & 1) {
+                                const double *a = c < 2 ? p0 : p1, *cc = cs + col + (c & 1);
+#pragma unroll 4
+                                for (int k = 0; k < p; ++k) f = fma(a[k], cc[k * q], f);
+                            }
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (u == c && (f64 >> u & 1)) v[u] = f;
+                        }
+                    }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
                         if (alpha != 1.0) v[c] = alpha == -1.0 ? -v[c] : alpha * v[c];
                         if (beta != 0.0) v[c] = (beta == 1.0 ? o[c] : beta * o[c]) + v[c];
                     }
@@ -517,7 +693,7 @@ int sm_count() {
 
 size_t nn_smem(int p, int q) {
     const int steps = (p + 15) / 16, ntiles = (q + 7) / 8;
-    return (size_t)ntiles * steps * kDigits * 32 * sizeof(uint2) + 2 * 64 * sizeof(int) + (size_t)p * q * sizeof(double);
+    return (size_t)ntiles * steps * (kDigits + 1) * 32 * sizeof(uint2) + 2 * 64 * sizeof(int) + (size_t)p * q * sizeof(double);
 }
 
 // row groups of one ts_tn launch: one warp per unit and group, a wave of blocks
