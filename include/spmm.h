@@ -233,8 +233,9 @@ typedef struct {
  * cudaHostRegister unless they are already pinned, and every spmm_apply
  * streams col_idx and values to HBM in blocks of whole warp tasks through two
  * staging slots (the copy of one block overlaps the multiplication of the
- * previous one).  A copy of row_ptr stays in HBM where 8 (n_rows + 3) bytes are
- * free; otherwise it is streamed as well.
+ * previous one).  row_ptr is streamed with them, or copied to HBM once where the
+ * handle then takes no more device memory than with row_ptr streamed (through
+ * stream_slot_kib slots, by default through 256 MiB ones).
  * The caller must keep the arrays alive and unchanged until spmm_destroy.
  * Only Y = A X is available; X and Y stay in HBM.  Calls on one streaming
  * handle share its slots and must not overlap.

@@ -9,8 +9,10 @@
 // X and Y stay in HBM, and the matrix flows over the host link in blocks of
 // whole warp tasks.  Two staging slots alternate: the copy of block b+1 runs
 // on a copy stream while the task kernel works on block b; events order each
-// slot's reuse.  The task list, row pointers, split table and partials live in
-// HBM as in the resident mode, so results are identical to it.
+// slot's reuse.  The task list, split table and partials live in HBM as in the
+// resident mode, so results are identical to it; the row pointers pass through
+// the slots like the rest, or stay in HBM where that takes no more memory
+// (stream_setup).
 //
 // The same pipeline serves a matrix kept in a file (spmm_create_file): each
 // block's column indices and values are first read from the file into one of
@@ -31,6 +33,7 @@ constexpr int64_t kSlotMinBytes = 16ll << 20, kSlotMaxBytes = 256ll << 20;
 // Cut the task list into blocks whose column-index range fits a slot.
 static void cut_blocks(const std::vector<int4>& tasks, int64_t n_rows, int64_t slot_nnz, std::vector<StreamBlock>& out,
                        int64_t* max_nnz, int64_t* max_rows) {
+    out.clear();
     auto e0 = [&](size_t t) { return ((int64_t)(uint32_t)tasks[t].z) | ((int64_t)tasks[t].w << 32); };
     const size_t nt = tasks.size() - 1;   // last descriptor is the sentinel
     *max_nnz = 0;
@@ -102,7 +105,17 @@ int stream_setup(spmm_mat* A, const int64_t* row_ptr, const int32_t* col_idx, co
                                    : std::min(kSlotMaxBytes, std::max(kSlotMinBytes, nnz * 4 / 8 + 4096));
     const int64_t slot_nnz = std::max<int64_t>(slot_bytes / 4, 2 * kMaxTaskNnz + 16);
     int64_t max_nnz = 0, max_rows = 0;
-    cut_blocks(plan.tasks, n, slot_nnz, S.blocks, &max_nnz, &max_rows);
+    // Row pointers in HBM save a ninth of the bytes of a matrix of 16 entries a row
+    // and one copy less per block (32 MB slots 1642 -> 1445 us).  But the memory of
+    // this mode is the dense matrices': they stay only where the handle then takes
+    // no more than with its row pointers streamed through the caller's slots or, by
+    // default, through the largest (256 MiB) ones: up to some 24 M rows of 16 entries
+    // by default, and matrices of one or two blocks with a slot of the caller's.
+    auto slots_bytes = [&](int64_t rows) { return 2 * ((max_nnz + 16) * (4 + (int64_t)vsize) + rows * 8); };
+    cut_blocks(plan.tasks, n, A->params.slot_bytes > 0 ? slot_nnz : kSlotMaxBytes / 4, S.blocks, &max_nnz, &max_rows);
+    const int64_t streamed_bytes = slots_bytes(max_rows + 4);
+    if (A->params.slot_bytes <= 0) cut_blocks(plan.tasks, n, slot_nnz, S.blocks, &max_nnz, &max_rows);
+    bool rp_in_hbm = slots_bytes(0) + (n + 3) * 8 <= streamed_bytes;
     S.slot_nnz = max_nnz + 16;
     S.slot_rows = max_rows + 4;
     cudaError_t e;
@@ -112,8 +125,6 @@ int stream_setup(spmm_mat* A, const int64_t* row_ptr, const int32_t* col_idx, co
         if (r == cudaSuccess) *bytes += (int64_t)b;
         return r;
     };
-    if (!S.h_rp_owned && (e = pin(row_ptr, (size_t)(n + 1) * 8, &S.reg_rp)) != cudaSuccess)
-        return cuda_fail(e, "streaming: pin row_ptr");
     if ((e = pin(col_idx, (size_t)nnz * 4, &S.reg_ci)) != cudaSuccess) return cuda_fail(e, "streaming: pin col_idx");
     if ((e = pin(values, (size_t)nnz * vsize, &S.reg_val)) != cudaSuccess) return cuda_fail(e, "streaming: pin values");
     for (int i = 0; i < 2; ++i) {
@@ -159,23 +170,30 @@ int stream_setup(spmm_mat* A, const int64_t* row_ptr, const int32_t* col_idx, co
             *bytes += (int64_t)d.n_slots * kSlotStride * sizeof(float);
         }
     }
-    // the row pointers stay in HBM (padded as in the resident mode): a ninth of the
-    // bytes of a matrix of 16 entries a row, and one copy less per block (32 MB
-    // slots 1642 -> 1445 us).  Unless what the rest leaves free is too little:
-    // then each block brings its own.
-    if (dmalloc((void**)&d.row_ptr, (size_t)(n + 3) * 8) == cudaSuccess) {
+    // the row pointers last: where the rest leaves too little they are streamed
+    if (rp_in_hbm && dmalloc((void**)&d.row_ptr, (size_t)(n + 3) * 8) != cudaSuccess) {
+        cudaGetLastError();
+        d.row_ptr = nullptr;
+        rp_in_hbm = false;
+    }
+    if (rp_in_hbm) {                       // padded as in the resident mode
         if ((e = cudaMemsetAsync(d.row_ptr + n + 1, 0, 16, s)) != cudaSuccess ||
             (e = cudaMemcpyAsync(d.row_ptr, row_ptr, (size_t)(n + 1) * 8, cudaMemcpyHostToDevice, s)) != cudaSuccess)
             return cuda_fail(e, "streaming: row pointers");
     } else {
-        cudaGetLastError();
-        d.row_ptr = nullptr;
+        if (!S.h_rp_owned && (e = pin(row_ptr, (size_t)(n + 1) * 8, &S.reg_rp)) != cudaSuccess)
+            return cuda_fail(e, "streaming: pin row_ptr");
         for (int i = 0; i < 2; ++i)
             if ((e = dmalloc((void**)&S.slot_rp[i], (size_t)S.slot_rows * 8)) != cudaSuccess)
                 return cuda_fail(e, "streaming: staging slots");
     }
     S.bytes_per_apply = nnz * 4 + (int64_t)(nnz * vsize) + (d.row_ptr ? 0 : (n + 1) * 8);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "streaming: set-up");
+    if (rp_in_hbm) {                       // nothing streams them: a file's pinned copy goes
+        S.h_row_ptr = nullptr;
+        cudaFreeHost(S.h_rp_owned);
+        S.h_rp_owned = nullptr;
+    }
     return SPMM_OK;
 }
 
