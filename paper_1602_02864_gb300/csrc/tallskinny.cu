@@ -49,7 +49,6 @@
 // the FP64 units alone would need about 7 ms.  What bounds them now is the
 // latency of the loads with 12 warps an SM (the mma take a quarter of the time).
 #include <algorithm>
-#include <mutex>
 
 #include <cuda_fp16.h>
 
@@ -728,12 +727,11 @@ cudaError_t ts_tn(const double* A, int64_t lda, int p, const double* B, int64_t 
 cudaError_t ts_nn(const double* A, int64_t lda, int p, const double* C, int q, double* Out, int64_t ldo, int64_t n,
                   double alpha, double beta, cudaStream_t s) {
     const size_t smem = nn_smem(p, q);
-    static std::once_flag once;
-    static cudaError_t setup = cudaSuccess;
-    std::call_once(once, [] {
-        setup = cudaFuncSetAttribute(ts_nn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nn_smem(64, 64));
-    });
-    if (setup != cudaSuccess) return setup;
+    // the attribute is the current device's: set where this launch needs it
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(ts_nn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     const int64_t rtiles = (n + 15) / 16;
     const unsigned grid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>((rtiles + kTsWarps - 1) / kTsWarps, sm_count()));
