@@ -784,7 +784,7 @@ static int apply_resident(const spmm_mat* A, int transpose, const void* X, int64
     a.compensated = d.partials_comp != nullptr || (A->params.compensated && d.n_slots == 0);
     a.partials_comp = d.partials_comp;
     a.ctl = d.ctl;
-    const bool combine_inside = combines_inside(d) && !a.compensated && !a.hot_cols;
+    const bool combine_inside = combines_inside(d, vmode, vec, ch, a.lanes_log2) && !a.compensated && !a.hot_cols;
     if (combine_inside) {         // a run holds all segments of its split rows
         a.splits = d.splits;
         a.n_splits = d.n_splits;
