@@ -332,13 +332,13 @@ __device__ __forceinline__ void issue_task(const FwdArgs& a, const int4 d0, int6
 // fits L2 (k = 16, 37 MB of X: 0.152 against 0.162 ms) and with two beyond
 // (134 MB: 0.836 against 0.569), narrower lanes always with two (k = 4, 67 MB
 // 0.510 against 0.433).
-template <int VMODE, int CH, bool ONE, int MG>
+template <int VMODE, int MG>
 constexpr bool two_blocks() {
     return (VMODE != 0 && MG == 0) || MG == 3 || MG == 4;
 }
-template <int VMODE, int CH, bool ONE, int MG>
+template <int VMODE, int MG>
 constexpr int min_blocks() {
-    return (MG == 2 && VMODE == 0) ? 4 : two_blocks<VMODE, CH, ONE, MG>() ? 2 : SPMM_MIN_BLOCKS;
+    return (MG == 2 && VMODE == 0) ? 4 : two_blocks<VMODE, MG>() ? 2 : SPMM_MIN_BLOCKS;
 }
 
 // *p counted up, wrapping to zero after `last`; everything before it is visible
@@ -419,7 +419,7 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     using Lay = Layout<VMODE>;
     // nonzeros in flight per lane group
     constexpr int kBytes = VEC * CH * (int)sizeof(XT);
-    constexpr bool kWide = MULTI || (two_blocks<VMODE, CH, ONE, MG>() && !HOT);
+    constexpr bool kWide = MULTI || (two_blocks<VMODE, MG>() && !HOT);
     constexpr int kU = SPMM_UNROLL_BYTES * (kWide ? 2 : 1) / kBytes;
     constexpr int U = kU < 2 ? 2 : (kU > 8 ? 8 : kU);
 #ifndef SPMM_MERGE_UNROLL
@@ -1158,7 +1158,7 @@ __device__ __forceinline__ void warp_done(const FwdArgs& ga, const MultiArgs* M)
 }
 
 template <typename XT, int VMODE, int VEC, int CH, bool COMP, bool ONE, int MG = 0, bool HOT = false, bool SEG = false>
-__global__ void __launch_bounds__(warps_per_block<HOT>() * 32, (HOT ? 1 : min_blocks<VMODE, CH, ONE, MG>()))
+__global__ void __launch_bounds__(warps_per_block<HOT>() * 32, (HOT ? 1 : min_blocks<VMODE, MG>()))
     rows_kernel(const __grid_constant__ FwdArgs a) {
     rows_run<XT, VMODE, VEC, CH, COMP, ONE, MG, HOT, false, SEG>(a, nullptr);
     if constexpr (self_reset<ONE, HOT, SEG>()) warp_done(a, nullptr);
@@ -1201,7 +1201,8 @@ cudaError_t launch_one(const FwdArgs& a, cudaStream_t s) {
         setup = e;
         num_sms = sms;
         max_smem = opt;
-        blocks_per_sm = nb > 0 ? nb : 1;
+        // two blocks even where the registers of a compiler's choice would let a third in
+        blocks_per_sm = nb < 1 ? 1 : (two_blocks<VMODE, MG>() && !HOT && nb > 2) ? 2 : nb;
     });
     if (setup != cudaSuccess) return setup;
     size_t smem = kStage;
@@ -1220,7 +1221,7 @@ cudaError_t launch_one(const FwdArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// One launch over the entries of M (generic row walk, three blocks per SM).
+// One launch over the entries of M (generic row walk, two blocks per SM).
 template <typename XT, int VMODE, int VEC, int CH, bool COMP>
 cudaError_t launch_multi_one(const MultiArgs& m, cudaStream_t s) {
     using Lay = Layout<VMODE>;
