@@ -432,7 +432,7 @@ def workload_streaming(args):
     (k = 4, FP32) in HBM; link bytes per call vs the measured pinned H2D peak."""
     import torch
     import oracle
-    from paper_1602_02864_gb300 import spmm
+    from paper_1602_02864_gb300 import probe, spmm
     scale = args.scale if args.scale != 24 else 29
     t = time.time()
     # the GPU generator makes the same graph as rmat_csr without a host-side edge sort
@@ -454,15 +454,19 @@ def workload_streaming(args):
     for _ in range(args.warmup):
         h.apply(X, Y=Y)
     # the host link can be shared with other jobs: time the streamed calls
-    # interleaved with a copy-only pass over the same host array (the column
-    # indices; the row pointers stay on the device with the handle)
-    ci = torch.from_numpy(A.col_idx).view(torch.uint8)
+    # interleaved with a copy-only pass over the same host arrays (the column
+    # indices and, unless the handle keeps them in HBM, the row pointers)
+    link_bytes = probe.spmm_probe_stream_bytes(h.handle)
+    sources = [torch.from_numpy(A.col_idx).view(torch.uint8)]
+    if link_bytes > nnz * 4:
+        sources.append(torch.from_numpy(A.row_ptr).view(torch.uint8))
     stage = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
 
     def copy_only():
-        for off in range(0, ci.numel(), 256 << 20):
-            n = min(256 << 20, ci.numel() - off)
-            stage[:n].copy_(ci[off:off + n], non_blocking=True)
+        for src in sources:
+            for off in range(0, src.numel(), 256 << 20):
+                n = min(256 << 20, src.numel() - off)
+                stage[:n].copy_(src[off:off + n], non_blocking=True)
     ms_list, copy_list = [], []
     for _ in range(args.steps):
         ms_list.append(event_ms(lambda: h.apply(X, Y=Y), 1))
@@ -473,7 +477,6 @@ def workload_streaming(args):
     peak_after = max((1 << 30) / (event_ms(lambda: dbuf2.copy_(buf2, non_blocking=True), 1) / 1e3) / 1e9
                      for buf2, dbuf2 in [(torch.empty(1 << 30, dtype=torch.uint8).pin_memory(),
                                           torch.empty(1 << 30, dtype=torch.uint8, device="cuda"))] for _ in range(5))
-    link_bytes = nnz * 4
     # resident mode on the same matrix for context
     hr = spmm.SparseMatrix(N, N, A.row_ptr, A.col_idx, None)
     Yr = torch.empty_like(Y)
@@ -499,7 +502,7 @@ def workload_streaming(args):
                                "frac_of_copy_only": copy_ms / ms,
                                "bytes_per_call": link_bytes,
                                "note": "steps alternate a streamed call and a copy-only pass over the same "
-                                       "pinned host array of column indices (the host link may be shared)"},
+                                       "pinned host arrays (the host link may be shared)"},
                       "resident_ms": ms_res, "bit_identical_to_resident": same,
                       "sampled_rows_max_err_over_absprod": err, "sampled_rows": int(len(rows)),
                       "n": N, "nnz": nnz, "setup_s": {"generate": round(t_gen, 1), "create": round(t_create, 1)}})
@@ -685,7 +688,7 @@ def workload_file(args):
     import tempfile
     import torch
     import oracle
-    from paper_1602_02864_gb300 import spmm
+    from paper_1602_02864_gb300 import probe, spmm
     N = 1 << args.scale
     A = synth.rmat_csr(args.scale, args.edge_factor * N, seed=0)
     nnz = A.nnz
@@ -723,7 +726,7 @@ def workload_file(args):
             ms = statistics.median(ts)
             entry[f"k{k}_ms"] = round(ms, 3)
             entry[f"k{k}_nnz_per_s"] = nnz / (ms / 1e3)
-            moved = nnz * 4 + ((N + 1) * 8 if name == "resident" else 0)    # other modes keep the row pointers in HBM
+            moved = probe.spmm_probe_stream_bytes(h.handle) or nnz * 4 + (N + 1) * 8
             entry[f"k{k}_matrix_GBps"] = moved / (ms / 1e3) / 1e9
         got = Y[8][torch.from_numpy(rows).cuda()].cpu().numpy()
         if ref is None:

@@ -98,6 +98,12 @@ __global__ void probe_cols_kernel(const int32_t* __restrict__ col, int64_t nnz, 
 
 using namespace spmm;
 
+extern "C" int spmm_probe_stream_bytes(spmm_mat_t A, int64_t* bytes) {
+    if (!A || !bytes) { set_error("spmm_probe_stream_bytes: NULL argument"); return SPMM_ERR_ARG; }
+    *bytes = A->streaming ? A->st.bytes_per_apply : 0;
+    return SPMM_OK;
+}
+
 extern "C" int spmm_probe_gather_cols(spmm_mat_t A, int32_t transpose, int32_t row_bytes, double* rows_per_s,
                                       double* bytes_per_s, void* stream) {
     if (!A || !rows_per_s || !bytes_per_s || row_bytes < 4 || row_bytes > 256 || row_bytes % 4) {

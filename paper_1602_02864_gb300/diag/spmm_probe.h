@@ -41,6 +41,14 @@ int spmm_probe_gather_cols(spmm_mat_t A, int32_t transpose, int32_t row_bytes, d
                            double* bytes_per_s, void* stream);
 
 /*
+ * spmm_probe_stream_bytes -- diagnostic: the bytes of A that each spmm_apply on
+ * a streaming handle copies from host memory or the file (column indices, values
+ * and, where the handle does not keep them in HBM, row pointers); 0 for a
+ * resident handle.
+ */
+int spmm_probe_stream_bytes(spmm_mat_t A, int64_t* bytes);
+
+/*
  * spmm_probe_ts_tn, spmm_probe_ts_nn -- diagnostic: the eigensolvers' FP64
  * products of tall, narrow matrices on device arrays, to check their accuracy
  * by themselves: C (p x q) = A^T B with A n x p, B n x q, and

@@ -19,6 +19,8 @@ _lib.spmm_probe_gather.argtypes = [_i64, _i32, _dp, _dp, _P]
 _lib.spmm_probe_gather.restype = ctypes.c_int
 _lib.spmm_probe_gather_cols.argtypes = [_P, _i32, _i32, _dp, _dp, _P]
 _lib.spmm_probe_gather_cols.restype = ctypes.c_int
+_lib.spmm_probe_stream_bytes.argtypes = [_P, ctypes.POINTER(_i64)]
+_lib.spmm_probe_stream_bytes.restype = ctypes.c_int
 _lib.spmm_probe_ts_tn.argtypes = [_P, _i64, _i32, _P, _i64, _i32, _i64, _P, _P]
 _lib.spmm_probe_ts_tn.restype = ctypes.c_int
 _lib.spmm_probe_ts_nn.argtypes = [_P, _i64, _i32, _P, _i32, _P, _i64, _i64, ctypes.c_double, ctypes.c_double, _P]
@@ -42,6 +44,13 @@ def spmm_probe_gather_cols(h, transpose, row_bytes, stream=None):
     _sp._check(_lib.spmm_probe_gather_cols(h, int(bool(transpose)), int(row_bytes), ctypes.byref(r),
                                            ctypes.byref(b), _sp._stream_handle(stream)))
     return r.value, b.value
+
+
+def spmm_probe_stream_bytes(h):
+    """Bytes of A that each product of a streaming handle copies (0: resident)."""
+    n = _i64(0)
+    _sp._check(_lib.spmm_probe_stream_bytes(h, ctypes.byref(n)))
+    return n.value
 
 
 def spmm_probe_ts_tn(A, B, C, stream=None):

@@ -27,6 +27,7 @@ def test_no_more_memory_than_streamed(sp, slot_kib, weighted):
     """Two slots of the block's column indices, values and row pointers, the task list and a page
     of counters: the bytes of a handle that streams its row pointers."""
     import torch
+    from paper_1602_02864_gb300 import probe
     n = 1 << 20
     rp, ci = long_and_thin(n)
     vals = np.random.default_rng(1).random(len(ci)).astype(np.float32) if weighted else None
@@ -41,6 +42,10 @@ def test_no_more_memory_than_streamed(sp, slot_kib, weighted):
         rows = min(n + 5, int(gaps.max()) + 128)
         allowed = 2 * (block * (8 if weighted else 4) + rows * 8) + 16 * (info["n_tasks"] + 1) + 4096
         assert info["device_bytes"] <= allowed
+        # streamed with a slot of the caller's, kept in HBM by default here
+        per_call = len(ci) * (8 if weighted else 4) + (8 * (n + 1) if slot_kib else 0)
+        assert probe.spmm_probe_stream_bytes(hs.handle) == per_call
+        assert probe.spmm_probe_stream_bytes(hr.handle) == 0
         for k in (1, 4, 33):
             X = torch.from_numpy(synth.dense(5000, k, seed=k)).cuda()
             Y = hr.apply(X)
