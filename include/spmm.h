@@ -23,8 +23,8 @@
  *     SPMM_RELABEL, a call that runs only A X products (spmm_apply,
  *     spmm_apply_host or spmm_apply_host_parts with transpose = 0) may
  *     overlap one that runs only A^T products (spmm_apply with transpose != 0,
- *     or spmm_pagerank): each orientation has its own task counter, scratch
- *     and hot-row buffer.  The host-buffer calls share the handle's group
+ *     or spmm_pagerank): each orientation has its own task counter and
+ *     scratch.  The host-buffer calls share the handle's group
  *     buffers, so two of them never overlap.  A host-buffer call that grows
  *     those buffers (the first, or one with wider groups) and a spmm_pagerank
  *     call that captures its graph (the first, or one with a new x, damping
@@ -382,8 +382,8 @@ int spmm_relabel_order(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
  * need (Section 3.4's single task queue over many multiplications): entries
  * whose X rows share a vector width and chunking (for float32 X: k = 8, 12,
  * ..., 64; k = 2, 4, 6, ...; k = 1 and odd k up to 31) run in one launch, their warp tasks
- * numbered one after the other; the split rows of all entries are combined
- * by one more launch.  Up to 128 entries share a launch; more make more
+ * numbered one after the other; a split row is added by the warp that brings
+ * its last segment.  Up to 128 entries share a launch; more make more
  * launches.  The entries' arguments travel in the kernels' parameter space,
  * so the call allocates nothing.
  *   n        number of entries (>= 1)
@@ -435,8 +435,8 @@ int spmm_write_csr_file(const char* path, int64_t n_rows, int64_t n_cols, int64_
  * spmm_create_file -- a handle whose matrix stays in a file written by
  * spmm_write_csr_file: the semi-external mode of Section 3.1 (vertex-sized
  * data in memory, edge-sized data on storage, streamed for every product).
- * The row pointers are read once into pinned host memory and the warp-task
- * plan goes to HBM; every spmm_apply reads the column indices (and values) of
+ * The row pointers are read once into pinned host memory (or HBM, by the rule of
+ * SPMM_HOST_STREAMING) and the warp-task plan goes to HBM; every spmm_apply reads the column indices (and values) of
  * each block of whole tasks from the file with parallel preads into pinned
  * staging buffers and streams them through two HBM slots as in
  * SPMM_HOST_STREAMING, so reading block b+1 overlaps copying and multiplying

@@ -1,8 +1,12 @@
-// combine.cu -- second pass for split (hub) rows in streaming mode, whose
-// launches each hold some of a row's segments (one launch over all of them adds
-// a row's partials itself): Y[row, :] = sum of the row's segment partials, added
-// in a fixed order so the result is the same on every run.  The partials of a call with k columns are packed k floats per slot
-// (slot s at s * k), so a small k reads only the floats it needs.
+// combine.cu -- second pass for split (hub) rows: Y[row, :] = sum of the row's
+// segment partials, added in a fixed order so the result is the same on every
+// run.  It serves streaming handles (whose launches each hold some of a row's
+// segments) and, on resident ones, task lists of more than kCombineInsideTasks,
+// compensated products, the hot variant, and pattern rows on 16 or more lanes of
+// one element (combines_inside, apply_resident); other launches, and the batched
+// ones, add a row's partials themselves.  The partials of a call with k columns
+// are packed k floats per slot (slot s at s * k), so a small k reads only the
+// floats it needs.
 #include "combine.cuh"
 
 namespace spmm {

@@ -1,6 +1,6 @@
 // combine.cuh -- the sum of a split row's segment partials, by one warp: the
 // last warp to finish a segment of the row (rows_kernel.cuh), or the combine
-// kernel where a row's segments are multiplied by several launches.
+// kernel (combine.cu, which says where).
 #pragma once
 
 #include "internal.h"

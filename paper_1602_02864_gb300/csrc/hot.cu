@@ -1,5 +1,5 @@
-// hot.cu -- the most-referenced columns of an orientation and their compact
-// copy of X.
+// hot.cu -- the most-referenced columns of an orientation and the column indices
+// that name them.
 //
 // The paper's largest compute gain comes from keeping the dense rows a tile
 // touches in cache (Section 3.4, Algorithm 1's tiles; Section 5.4 cache
@@ -11,10 +11,11 @@
 // (k = 1 float32, k = 2 bf16/f16) runs the hot variant (one block of 24 warps
 // per SM), whose blocks gather the H hot rows of X into shared memory at their
 // start and read them from there, so only the other gathers use the L1-to-L2
-// request path, which bounds the k = 1 product (78% busy on R-MAT).  The 8192 hottest columns take 21% of
-// R-MAT scale 24's entries; the product runs 10% faster with them (the
-// shared memory they take is L1 that the other gathers lose).  The sums and
-// their order are unchanged: only the address a row is read from differs.
+// request path, which bounds the k = 1 product (78% busy on R-MAT without hot rows).  The
+// 8192 hottest columns take 21% of R-MAT scale 24's entries; the product runs 10%
+// faster with them (the shared memory they take is L1 that the other gathers
+// lose).  The sums and their order are unchanged: only the address a row is read
+// from differs.
 #include <algorithm>
 #include <functional>
 #include <numeric>

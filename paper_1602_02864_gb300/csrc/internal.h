@@ -29,8 +29,9 @@ struct NvtxRange {
 //   x >= 1 : a run of x short rows r0 .. r0+x-1 (one lane group per row)
 //   x == 0 : one long row r0 (all lane groups share its nonzeros)
 //   x < 0  : one segment of a split hub row r0; its partial result goes to
-//            slot -x-1 and combine.cu adds the segments in order.
-//   split  = int4 {row, nseg, slot0, 0} for the combine pass.
+//            slot -x-1, and the segments are added in order by the warp that
+//            brings the last one or by a second launch (combines_inside).
+//   split  = int4 {row, nseg, slot0, 0} for that sum.
 constexpr int kWarpsPerBlock = 8;
 constexpr int kMaxTaskNnz = 512;    // staged nonzeros per task (shared memory)
 constexpr int kMaxTaskRows = 64;    // rows per short-row task
@@ -394,7 +395,10 @@ struct FwdArgs {
 
 // X beyond the part of L2 that random gathers fill (64 MB of the GPU's L2: uniform
 // gathers of 32-byte rows run at 304 G rows/s from a 64 MB table, 125 from
-// 128 MB, 76 from 256 MB).
+// 128 MB, 76 from 256 MB).  For the weighted group merge (rows_*_mg.cu) the two
+// forms cross between 50 and 72 MB, by type and width (us with three / two blocks a
+// SM: FP32 k = 12, 50 MB of X 182 / 174, 62 MB 236 / 211; k = 16, 64 MB 181 / 176,
+// 74 MB 200 / 188; BF16 k = 12, 50 MB 313 / 338, 72 MB 476 / 476, 101 MB 664 / 652).
 constexpr int64_t kLargeXBytes = 64ll << 20;
 
 // One launch over the tasks of several matrices (spmm_apply_batched): the

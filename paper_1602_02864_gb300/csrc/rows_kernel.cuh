@@ -432,7 +432,10 @@ __device__ __forceinline__ void rows_run(const FwdArgs& ga, const MultiArgs* M) 
     // merge over lane groups: nonzeros in flight per group.  Values are read from
     // shared memory when they are used and the task state fits few registers, so
     // 4 in flight spill neither with values (2 before: k = 16 weighted, 37 MB of
-    // X 0.168 -> 0.152 ms) nor without; 6 do (0.211).
+    // X 0.168 -> 0.152 ms) nor without; 6 do (0.211).  The compensated form over
+    // 16-byte lanes spills 60 bytes and is as fast as with 2 (k = 16, 1 M vertices
+    // 256 us, 262).  Four blocks (MG == 2) spill 92 bytes with 2 in flight and 112 in
+    // the form that adds split rows; min_blocks()'s figures have that in them.
     constexpr int kUW = MG == 4   ? 8
                         : MG == 3 ? 2 * SPMM_MERGE_WIDE_UNROLL
                         : MG == 1 ? SPMM_MERGE_WIDE_UNROLL

@@ -43,11 +43,17 @@
 // different size 4.9e-16 -> 2.0e-16, power-law rows 3.3e-16 -> 6.9e-17; A C, 2-norm
 // of the error, 4.6e-17 -> 9.3e-18, 8.7e-16 -> 1.6e-16, 5.1e-16 -> 8.6e-17.
 // Digits are made with integer instructions only, since conversions to and from
-// FP64 run at the rate of the FP64 units.  Measured, one restart of the block
-// Krylov-Schur solver on 148,444 vertices (basis 64, block 16; 26 products of each
-// kind): A^T B 8.5 -> 1.3 ms, A C 3.8 -> 1.6 ms, reductions of partials 0.73 -> 0.37 ms;
-// the FP64 units alone would need about 7 ms.  What bounds them now is the
-// latency of the loads with 12 warps an SM (the mma take a quarter of the time).
+// FP64 run at the rate of the FP64 units.  Measured, two cycles of the block
+// Krylov-Schur solver (one restart) on 148,444 vertices, basis 64, block 16, the
+// sums of their launches: A^T B 8.5 -> 1.7 ms (1.3 without the magnitudes' pass),
+// A C 3.8 -> 2.0 ms (W R^-1 in FP64 arithmetic included, 0.5 ms of it; 1.6 with
+// digits throughout), reductions of partials 0.73 -> 0.37 ms; the FP64 units alone
+// would need about 7 ms.  The elements below the line cost up to as much as the digits of
+// their product: V C of the first Gram-Schmidt pass 76 -> 139 us (32 columns), 93 -> 148
+// (48).  Neither memory (DRAM 5-13%, L2 6%) nor the tensor pipe (8-24%) bounds these
+// kernels: with 12 warps an SM (168 registers) they issue on 27-48% of the cycles and
+// wait on fixed latencies, loads and the tensor pipe in about equal parts (ts_tn), on
+// FP64 results and shared memory where elements fall back (ts_nn).
 #include <algorithm>
 
 #include <cuda_fp16.h>
