@@ -312,9 +312,9 @@ int apply_dev_runs(const spmm_mat* A, int transpose, const void* X, int64_t ldx,
 // waits for its stores and an atomic; a second launch costs 2-3 us (R-MAT, k = 8
 // weighted: 406 tasks, 4 K vertices 12.5 -> 8.7 us; 5,002 tasks, 64 K 21.9 ->
 // 18.3; k = 1 15.8 -> 12.7; but k = 8, 512 K vertices, 36,046 tasks 67.7 ->
-// 70.8, 4 M vertices 400 -> 475).  Around the line the two are within 5% of each
-// other either way (13,800 to 18,000 tasks: pattern k = 16 58.6 -> 53.5 us, k = 64 111 ->
-// 115).  Not for pattern rows on 16 or more lanes of one element, whose kernel
+// 70.8, 4 M vertices 400 -> 475).  Near the line it depends on the width (11,300
+// tasks, pattern k = 16 49.7 -> 45.3 us, k = 64 92.7 -> 95.1; 19,000 tasks 58.6 -> 53.5,
+// 111 -> 115).  Not for pattern rows on 16 or more lanes of one element, whose kernel
 // loses more to the arrivals' registers than the launch costs (FP32 outside / inside:
 // k = 13, 64 K vertices 48.8 / 54.2, 128 K 64.8 / 75.3; k = 31 68.9 / 77.4, 95 / 108;
 // BF16 k = 31 70.2 / 77.0; k = 5 on 8 lanes 40.2 / 35.7).

@@ -34,9 +34,10 @@
 // many products: the error bound of each element is that of FP64 arithmetic,
 // whatever the data.  FP64 arithmetic also takes the elements whose columns (rows)
 // hold subnormal numbers or whose scales are near the ends of the exponent range.
-// Share of the elements below the line, block Krylov-Schur on a symmetrised R-MAT
-// graph: A^T B 0.01%, the subtraction of V C 3%, Ritz vectors none; W R^-1 would
-// have 3-14%, and stays in FP64 arithmetic (eigs.cu).
+// Share of the elements that do, block Krylov-Schur on a symmetrised R-MAT graph,
+// first cycles / converged: A^T B below 0.01% / 0.6%, the subtraction of V C none,
+// Ritz vectors none / 0.2%.  W R^-1 would have up to 13%, and a kernel for triangular
+// factors is as fast in FP64 arithmetic (eigs.cu).
 // A tile (row) with an infinity or a NaN gives NaN.
 // Largest error against quadruple precision, FP64 kernels -> digits: A^T B,
 // 20,000 x 48 by 16, orthonormal columns 7.7e-18 -> 4.9e-18, with rows of very
@@ -443,9 +444,15 @@ __global__ void __launch_bounds__(256) ts_reduce_kernel(const double* __restrict
 // in CholQR); then every column of C is scaled by its largest element.  The
 // digits of C sit in shared memory in fragment order (made once per block); a
 // warp takes 16 rows of A at a time and for each 16 columns of Out multiplies
-// the digits of up to 64 columns of A into one set of accumulators.  With Out
-// added unscaled, an element of Out that is larger than what could be left out
-// times 2^53 hides it in the last rounding, and needs no FP64 arithmetic.
+// the digits of up to 64 columns of A into one set of accumulators.
+// The largest element of each column of C is left out of the digits and its
+// product added by one FP64 multiply-add: C is often near a diagonal matrix (the
+// Ritz vectors once they converge, V^T W of a restarted cycle), so that an element of
+// Out is about one element of A, often far below its row's largest, and the digits
+// then hold only the small rest.  An element takes FP64 arithmetic only if neither
+// its sum of magnitudes nor that largest product is above the line; with Out added
+// unscaled, an element of Out that is larger than what could be left out times 2^53
+// hides it too.
 __global__ void __launch_bounds__(kTsWarps * 32, 1)
 ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __restrict__ C, int q, double* Out,
              int64_t ldo, int64_t n, double alpha, double beta, int vec2) {
@@ -455,8 +462,20 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
     uint2* cb = cd + (int64_t)ntiles * steps * kDigits * 32;                         // [ntile][step][lane]: magnitudes
     int* ce = reinterpret_cast<int*>(cb + (int64_t)ntiles * steps * 32);             // exponent of column j of C
     int* cr = ce + 64;                                                               // exponent of row k of C - 1023
-    double* cs = reinterpret_cast<double*>(cr + 64);                                 // C
+    int* cp = cr + 64;                                                               // row of column j's largest element
+    double* cs = reinterpret_cast<double*>(cp + 64);                                 // C
     for (int i = threadIdx.x; i < p * q; i += blockDim.x) cs[i] = C[i];
+    __syncthreads();
+    for (int j = threadIdx.x; j < 64; j += blockDim.x) {
+        uint32_t h = 0;
+        int row = 0;
+        if (j < q)
+            for (int k = 0; k < p; ++k) {
+                const uint32_t x = magnitude(cs[k * q + j]);
+                if (x > h) h = x, row = k;
+            }
+        cp[j] = row;
+    }
     __syncthreads();
     bool sub = false;                                // a subnormal element of C
     for (int k = threadIdx.x; k < 64; k += blockDim.x) {
@@ -464,7 +483,7 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
         if (k < p)
             for (int j = 0; j < q; ++j) {
                 const uint32_t x = magnitude(cs[k * q + j]);
-                h = max(h, x);
+                if (cp[j] != k) h = max(h, x);
                 sub |= x != 0 && (x >> 20) == 0;
             }
         cr[k] = (h >> 20) == 0 ? kNoExp : (int)(h >> 20) - 1023;
@@ -478,6 +497,7 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
                 const uint32_t h = magnitude(cs[k * q + j]);
                 const int x = (int)(h >> 20);
                 special |= x == 0x7ff;
+                if (cp[j] == k) continue;
                 zero &= h == 0;
                 if (x > 0) e = max(e, x - cr[k]);
             }
@@ -492,7 +512,7 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int k = ks * 16 + 2 * t + (r & 1) + (r >> 1) * 8;
-            const double c = k < p && col < q ? cs[k * q + col] : 0.0;
+            const double c = k < p && col < q && k != cp[col] ? cs[k * q + col] : 0.0;
             y[r] = digits_of(c, ce[col] + cr[k]);
             m[r] = bf16_below(magnitude(c), ce[col] + cr[k]);
         }
@@ -626,24 +646,45 @@ ts_nn_kernel(const double* __restrict__ A, int64_t lda, int p, const double* __r
                     uint32_t f64 = fp64 >> (4 * (np + j)) & 15u;
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        const int e = c < 2 ? e0 : e1, ec = ce[col + (c & 1)];
-                        v[c] = from_diagonals(acc[j], c, e, ec);
-                        if (hides && !c_sub && !(c < 2 ? sub0 : sub1) && (int)(magnitude(o[c]) >> 20) >= e + ec - hidden &&
-                            e + ec >= 1090 && e + ec <= 3061)
+                        const int e = c < 2 ? e0 : e1, ec = ce[col + (c & 1)], top = cp[col + (c & 1)];
+                        const double a = (c < 2 ? p0 : p1)[top], d = cs[top * q + min(col + (c & 1), q - 1)];
+                        v[c] = fma(a, d, from_diagonals(acc[j], c, e, ec));
+                        // hidden behind the largest product (or a zero factor, exponent field 0: not), or behind Out
+                        const int xa = (int)(magnitude(a) >> 20), xd = (int)(magnitude(d) >> 20);
+                        if (!c_sub && !(c < 2 ? sub0 : sub1) && e + ec >= 1090 && e + ec <= 3061 &&
+                            ((xa > 0 && xd > 0 && xa + xd >= e + ec - 3) ||
+                             (hides && (int)(magnitude(o[c]) >> 20) >= e + ec - hidden)))
                             f64 &= ~(1u << c);
                     }
-                    if (__any_sync(0xffffffffu, f64 != 0)) {
-#pragma unroll 1
-                        for (int c = 0; c < 4; ++c) {
-                            double f = 0.0;
-                            if (f64 >> c & 1) {
-                                const double *a = c < 2 ? p0 : p1, *cc = cs + col + (c & 1);
-#pragma unroll 4
-                                for (int k = 0; k < p; ++k) f = fma(a[k], cc[k * q], f);
-                            }
+                    // the warp's elements in need, one a lane: the FP64 units take as long for one as for 32
+                    uint32_t need[4];
+                    int first[5] = {0, 0, 0, 0, 0};
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (u == c && (f64 >> u & 1)) v[u] = f;
+                    for (int c = 0; c < 4; ++c) {
+                        need[c] = __ballot_sync(0xffffffffu, f64 >> c & 1);
+                        first[c + 1] = first[c] + __popc(need[c]);
+                    }
+#pragma unroll 1
+                    for (int base = 0; base < first[4]; base += 32) {
+                        const int i = base + lane;
+                        double f = 0.0;
+                        if (i < first[4]) {
+                            int c = 0;
+                            uint32_t mask = need[0], nth = i + 1;
+#pragma unroll
+                            for (int u = 1; u < 4; ++u)
+                                if (i >= first[u]) c = u, mask = need[u], nth = i - first[u] + 1;
+                            const int src = __fns(mask, 0, nth);         // the lane whose element it is
+                            const double* a = A + (rt * 16 + (src >> 2) + (c < 2 ? 0 : 8)) * lda;
+                            const double* cc = cs + (np + j) * 8 + 2 * (src & 3) + (c & 1);
+#pragma unroll 4
+                            for (int k = 0; k < p; ++k) f = fma(a[k], cc[k * q], f);
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int at = first[u] + __popc(need[u] & ((1u << lane) - 1u)) - base;
+                            const double mine = __shfl_sync(0xffffffffu, f, at & 31);
+                            if ((f64 >> u & 1) && at >= 0 && at < 32) v[u] = mine;
                         }
                     }
 #pragma unroll
@@ -698,7 +739,7 @@ int sm_count() {
 
 size_t nn_smem(int p, int q) {
     const int steps = (p + 15) / 16, ntiles = (q + 7) / 8;
-    return (size_t)ntiles * steps * (kDigits + 1) * 32 * sizeof(uint2) + 2 * 64 * sizeof(int) + (size_t)p * q * sizeof(double);
+    return (size_t)ntiles * steps * (kDigits + 1) * 32 * sizeof(uint2) + 3 * 64 * sizeof(int) + (size_t)p * q * sizeof(double);
 }
 
 // row groups of one ts_tn launch: one warp per unit and group, a wave of blocks
