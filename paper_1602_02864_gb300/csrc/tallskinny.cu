@@ -47,14 +47,13 @@
 // FP64 run at the rate of the FP64 units.  Measured, two cycles of the block
 // Krylov-Schur solver (one restart) on 148,444 vertices, basis 64, block 16, the
 // sums of their launches: A^T B 8.5 -> 1.7 ms (1.3 without the magnitudes' pass),
-// A C 3.8 -> 2.0 ms (W R^-1 in FP64 arithmetic included, 0.5 ms of it; 1.6 with
-// digits throughout), reductions of partials 0.73 -> 0.37 ms; the FP64 units alone
-// would need about 7 ms.  The elements below the line cost up to as much as the digits of
-// their product: V C of the first Gram-Schmidt pass 76 -> 139 us (32 columns), 93 -> 148
-// (48).  Neither memory (DRAM 5-13%, L2 6%) nor the tensor pipe (8-24%) bounds these
-// kernels: with 12 warps an SM (168 registers) they issue on 27-48% of the cycles and
-// wait on fixed latencies, loads and the tensor pipe in about equal parts (ts_tn), on
-// FP64 results and shared memory where elements fall back (ts_nn).
+// A C 3.8 -> 1.9 ms (0.5 of it W R^-1 in FP64 arithmetic; 1.6 with digits throughout
+// and no guard), reductions of partials 0.73 -> 0.37 ms; the FP64 units alone would
+// need about 7 ms.  Neither memory (DRAM 7-14%, L2 6%) nor the tensor pipe (9-24%)
+// bounds these kernels: with 12 warps an SM (168 registers) they issue on 35-51% of
+// the cycles.  A warp of ts_tn waits on fixed latencies, loads and the tensor pipe in
+// about equal parts; one of ts_nn on fixed latencies and on shared memory and FP64
+// results, the FP64 pipe being 31-46% busy with the additions into Out.
 #include <algorithm>
 
 #include <cuda_fp16.h>
