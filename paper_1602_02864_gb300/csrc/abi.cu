@@ -78,7 +78,12 @@ static cudaError_t upload(T** dst, const T* src, size_t count, size_t pad, cudaS
 // each split row, on the device.
 static cudaError_t upload_split_state(const HostPlan& plan, int2** slot_seg, unsigned int** seg_done, cudaStream_t s,
                                       int64_t* bytes) {
-    std::vector<int2> of((size_t)plan.n_slots);
+    std::vector<int2> of;
+    try {
+        of.resize((size_t)plan.n_slots);
+    } catch (const std::bad_alloc&) {           // a C entry lets no exception out
+        return cudaErrorMemoryAllocation;
+    }
     for (size_t i = 0; i < plan.splits.size(); ++i)
         std::fill_n(of.begin() + plan.splits[i].z, plan.splits[i].y, make_int2((int)i, plan.splits[i].y));
     cudaError_t e = upload(slot_seg, of.data(), of.size(), 0, s, bytes);
